@@ -91,11 +91,13 @@ typedef struct lsweep_params {
   int maxit;          /* maximum preconditioner applications per solve (default 500)  */
   double tol;         /* relative residual ||f - A u|| / ||f|| to reach (default 1e-8)*/
   void* stream;       /* cudaStream_t to issue work on; NULL = the default stream     */
-  int front_kernel;   /* sweep-front kernel: 0 automatic (default: 3 where it applies),  */
-                      /* 1 cluster-split row slabs (any b), 2 one CTA per solve          */
-                      /* streaming whole blocks, 3 two CTAs per solve on a factor        */
-                      /* twisted at the middle line (each CTA eliminates from one end;   */
-                      /* 2 and 3: complex64, line width b <= 92 only)                    */
+  int front_kernel;   /* sweep-front kernel: 0 automatic (default: the twisted kernels where */
+                      /* they apply: 2D lines of up to about 146 nodes in complex64, 100 in */
+                      /* complex128), 1 cluster-split row slabs (any b), 2 one CTA per      */
+                      /* solve streaming whole blocks, 3 the twisted kernels: a cluster per */
+                      /* solve on a factor twisted at the middle line, each half            */
+                      /* eliminating from one end, the symmetric block inverses stored as   */
+                      /* triangles (2 and 3: complex64, line width b <= 92 only)            */
   int prefetch_steps; /* kernels 2, 3: steps of bulk L2 prefetch ahead of the block      */
                       /* stream; planes too wide for a row slab per ring slot (3D): row  */
                       /* chunks between a ring copy and the L2 prefetch it issues        */
@@ -224,10 +226,11 @@ int lsweep_update_m(lsweep_handle h, const double* m_bulk);
 
 /* Phase 2 "Factorize" (Sec. 3): block-tridiagonal LU of every local matrix over its grid
  * lines (2D) or planes (3D), storing the dense inverse Schur complements
- * D_k^-1, D_k = A_kk - L_k D_{k-1}^-1 U_{k-1}, in the handle's precision.  With sweep-front
- * kernel 3 (the complex64 default where it applies) the factor is twisted at the middle line
+ * D_k^-1, D_k = A_kk - L_k D_{k-1}^-1 U_{k-1}, in the handle's precision.  With the twisted
+ * kernels (the 2D default where they apply) the factor is twisted at the middle line
  * m = (L - 1) / 2: lines 0..m-1 are eliminated from line 0, lines L-1..m+1 from line L-1, and
- * block m inverts the Schur complement that takes both neighbours' updates.  Returns
+ * block m inverts the Schur complement that takes both neighbours' updates; of each inverse,
+ * symmetric as the operator is, the triangle is stored.  Returns
  * LSWEEP_ESINGULAR if a block had a zero or non-finite pivot.  Synchronous. */
 int lsweep_factor(lsweep_handle h);
 
@@ -299,7 +302,7 @@ int lsweep_solve_batch(int nprob, const lsweep_handle* hs, const void* const* f,
  * lsweep_solve_batch's.  Arguments as for lsweep_solve_batch.  The handles must be
  * complex64, right-preconditioned FGMRES, without windows, and share the sweep-front
  * geometry (line width, padded width, line count: equal subdomain widths and PML) and form
- * (twisted factors with two CTAs per solve, or one CTA per solve); LSWEEP_EINVAL with a
+ * (twisted factors, or one CTA per solve); LSWEEP_EINVAL with a
  * message on the first handle otherwise.  The Arnoldi work of each problem runs on its
  * handle's stream.  Synchronous. */
 int lsweep_solve_batch_fused(int nprob, const lsweep_handle* hs, const void* const* f,
@@ -381,10 +384,12 @@ int lsweep_local_shape(lsweep_handle h, int i, int j, int shape[3], int origin[3
 /* Number of extended-grid nodes N_e^dim (host output). */
 int lsweep_ext_size(lsweep_handle h, int64_t* n_ext);
 
-/* Bytes of the stored factors, and the factor bytes one lsweep_apply streams with the
- * sweep-front kernel in use (after lsweep_factor): per dependency level and subdomain,
- * 2 L b^2 element sizes less the forward block steps over lines where the right-hand side
- * is zero, which the complex64 one- and two-CTA kernels skip.  Host outputs. */
+/* Bytes of the stored factors, and the factor bytes of one lsweep_apply with the sweep-front
+ * kernel in use (after lsweep_factor) counted in whole blocks: per dependency level and
+ * subdomain, 2 L b^2 element sizes less the block steps that the kernel skips (forward over
+ * lines where the right-hand side is zero: one-CTA and twisted kernels; backward past the last
+ * line that is read: twisted kernels).  Twisted factors store and stream the triangle of each
+ * block, (b + 1) / (2 b) of this (lsweep_profile.front_bytes).  Host outputs. */
 int lsweep_factor_bytes(lsweep_handle h, int64_t* stored, int64_t* per_apply);
 
 /* Result of lsweep_autotune (host struct). */
@@ -397,7 +402,7 @@ typedef struct lsweep_tuning {
 
 /* Choose the sweep-front kernel and its L2 prefetch distance for this handle's plan by
  * timing `trials` applications of each configuration the widest line admits (the
- * two-CTA kernel on the twisted factor with prefetch 0, 2, 4; the one-CTA-per-solve kernel
+ * twisted kernels with prefetch 0, 2, 4; the one-CTA-per-solve kernel
  * with prefetch 0, 2, 4, 8; the cluster split), and keep the fastest in the handle's
  * parameters.  Moving between the twisted and the plain factor refactors the handle (while
  * clones share its factors, only kernels of the current factor form are tried).  Needs a
@@ -424,7 +429,8 @@ typedef struct lsweep_profile {
                             /* application replayed from a CUDA graph is timed as a whole,*/
                             /* its trace reset and lane sum included)                     */
   double front_bytes;       /* factor bytes those launches must stream: per subdomain      */
-                            /* visited, 2 L b^2 element sizes (forward and backward)       */
+                            /* visited, forward and backward, whole blocks of b^2 entries  */
+                            /* or (twisted factors) their triangles, skipped steps left out */
   double factor_ms;         /* duration of the last lsweep_factor (CUDA events)           */
 } lsweep_profile;
 

@@ -513,14 +513,17 @@ int build_plan(Ctx* c) {
       for (int f = 0; f < 3; ++f)
         nblk[f][at] = std::max(nblk[f][at], lsw::solve_blocks(g, x.kind, c->dim, f));
     }
+    // per_apply counts whole b x b blocks; the bytes of a launch are those of the storage the
+    // kernel streams (twisted factors: the triangle)
     for (int f = 0; f < 3; ++f) {
-      long long le = 0;
+      long long le = 0, st = 0;
       for (size_t u = 0; u < seen.size(); ++u) {
         const auto& g = c->subs[seen[u]];
         le += (long long)nblk[f][u] * g.b * (long long)g.b;
+        st += (long long)nblk[f][u] * (f == 2 ? g.b * (g.b + 1LL) / 2 : g.b * (long long)g.b);
       }
       c->per_apply_elems_f[f] += le;
-      c->launch_bytes_f[f].push_back((double)le * c->welem());
+      c->launch_bytes_f[f].push_back((double)st * c->welem());
     }
   }
   return LSWEEP_OK;
@@ -1265,7 +1268,13 @@ int lsweep_ext_size(lsweep_handle h, int64_t* n_ext) {
 int lsweep_factor_bytes(lsweep_handle h, int64_t* stored, int64_t* per_apply) {
   Ctx* c = (Ctx*)h;
   if (!c || !stored || !per_apply) return LSWEEP_EINVAL;
-  *stored = c->fac_elems * (int64_t)c->welem();
+  int64_t elems = c->fac_elems;
+  if (c->twisted()) {
+    elems = 0;
+    const lsw::TileStore st = lsw::tile_store(*c);
+    for (const auto& g : c->subs) elems += (int64_t)g.L * lsw::block_elems(g.b, st);
+  }
+  *stored = elems * (int64_t)c->welem();
   *per_apply = c->per_apply_elems_f[lsw::front_form(*c)] * (int64_t)c->welem();
   return LSWEEP_OK;
 }
@@ -1299,7 +1308,7 @@ std::vector<TuneCand> tune_candidates(Ctx* c) {
   std::vector<TuneCand> cands;
   const lsweep_params saved = c->p;
   const bool tw0 = c->fac_twisted;
-  for (int pd : {0, 2}) {   // automatic: two CTAs per solve, four on levels of few solves
+  for (int pd : {0, 2}) {   // automatic
     c->p.front_kernel = 0;
     c->p.prefetch_steps = pd;
     if (lsw::wants_twisted(*c) && (c->clones == 0 || tw0)) cands.push_back({0, pd});
@@ -1433,7 +1442,7 @@ int lsweep_autotune(lsweep_handle h, int trials, lsweep_tuning* out) {
   if (trials < 1 || trials > 100) return fail(c, LSWEEP_EINVAL, "trials must be in [1, 100]");
   if (c->profiling) return fail(c, LSWEEP_EINVAL, "switch profiling off before tuning");
   const lsweep_params saved = c->p;
-  // candidates that the plan's widest line admits; the two-CTA kernel needs twisted factors
+  // candidates that the plan's widest line admits; the twisted kernels need twisted factors
   // and the others plain ones, so switching between them refactors (not while clones share
   // the factors: then only the current form is tried)
   std::vector<TuneCand> cands = tune_candidates(c);

@@ -26,7 +26,7 @@ namespace lsw {
 // Stored block k holds the inverse of line k's Schur complement and the couplings c_k, c_{k-1}.
 template <typename C>
 __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restrict__ lcoef,
-                              long long cstride, C* __restrict__ fac, int dim, int twisted,
+                              long long cstride, C* __restrict__ fac, int dim, TileStore ts,
                               int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SubGeom g = subs[blockIdx.x];
@@ -40,6 +40,7 @@ __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restr
   const C* cy = d + 2 * cstride;
   const C* cl = dim == 3 ? d + 3 * cstride : cy;   // coupling between consecutive lines
   const int tid = threadIdx.x, nth = blockDim.x;
+  const bool twisted = ts.T > 0;
   const int m = twisted ? twist_line(L) : L;
   for (int st = 0; st < L; ++st) {
     // line k; coupling line ci of the update by the inverse held in M (the previous line's),
@@ -56,7 +57,8 @@ __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restr
       if (m < L - 1) ci = m;
       if (m > 0) cg = m - 1;
     }
-    const C* Dg = fac + g.fac_off + (long long)(cg < 0 ? 0 : cg) * g.bs;
+    const long long bstr = twisted ? block_elems(b, ts) : g.bs;
+    const C* Dg = fac + g.fac_off + (cg < 0 ? 0 : cg) * bstr;
     // Schur complement of line k, built in place over the previous inverse
     for (int idx = tid; idx < b * b; idx += nth) {
       int col = idx / b, row = idx - col * b;
@@ -73,13 +75,42 @@ __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restr
       }
       if (cg >= 0) {
         C lr = cl[(size_t)cg * b + row], lc = cl[(size_t)cg * b + col];
-        v = v - cmul(cmul(lr, Dg[(size_t)row * bp + col]), lc);
+        v = v - cmul(cmul(lr, Dg[tile_index(b, ts, (int)sizeof(C), row, col)]), lc);
       }
       M[(size_t)col * bp + row] = v;
     }
     __syncthreads();
     gauss_jordan_inverse<C>(M, b, bp, f, prow, perm, status);
-    C* Dk = fac + g.fac_off + (long long)k * g.bs;
+    C* Dk = fac + g.fac_off + k * bstr;
+    if (twisted) {
+      // the tiles of the symmetric part, which replaces the inverse in M as well: the next
+      // line's Schur complement is then that of the stored block.  n: b padded to whole tiles
+      const int n = tile_rows(b, ts.T) * ts.T;
+      for (int idx = tid; idx < n * (n + 1) / 2; idx += nth) {
+        // pair idx of the triangle, two columns of it folded into one of n + 1 entries
+        const int j = idx / (n + 1), i = idx - j * (n + 1);
+        const int row = i > j ? i - 1 : n / 2 + j, col = i > j ? j : n / 2 + i;
+        C v = czero<C>();
+        if (row < b) {
+          const C u = M[(size_t)col * bp + row], t = M[(size_t)row * bp + col];
+          v = mk((u.x + t.x) / 2, (u.y + t.y) / 2);
+          M[(size_t)col * bp + row] = v;
+          M[(size_t)row * bp + col] = v;
+        }
+        Dk[tile_index(b, ts, (int)sizeof(C), row, col)] = v;
+      }
+      const int bs = (b + 1) & ~1;
+      for (int q = 0; q < ts.NQ; ++q) {
+        C* part = Dk + (q ? part_elems(b, ts, 0) : 0);
+        const int c0 = part_cpl(b, ts, q);
+        for (int p = tid; p < 2 * bs; p += nth) {
+          const int up = p >= bs, col = up ? p - bs : p, kk = k - up;   // c_k, then c_{k-1}
+          part[c0 + p] = col < b && kk >= 0 ? cl[(size_t)kk * b + col] : czero<C>();
+        }
+      }
+      __syncthreads();
+      continue;
+    }
     for (int idx = tid; idx < g.bs; idx += nth) {
       int row = idx / bp, col = idx - row * bp;
       C v = czero<C>();
@@ -408,7 +439,7 @@ cudaError_t launch_factor(Ctx& c) {
     if (e != cudaSuccess) return e;
     k_factor_simt<float2><<<nsub, th, smem, c.stream>>>(c.d_subs, (const float2*)c.d_lcoef,
                                                         c.node_elems, (float2*)c.d_fac, c.dim,
-                                                        c.fac_twisted ? 1 : 0, c.d_status);
+                                                        c.fac_twisted ? tile_store(c) : TileStore{0, 1}, c.d_status);
   } else {
     size_t smem = (size_t)c.bpmax * c.bmax * sizeof(double2) + 2 * c.bmax * sizeof(double2) +
                   c.bmax * sizeof(int) + 16;
@@ -417,7 +448,7 @@ cudaError_t launch_factor(Ctx& c) {
     if (e != cudaSuccess) return e;
     k_factor_simt<double2><<<nsub, th, smem, c.stream>>>(c.d_subs, (const double2*)c.d_lcoef,
                                                          c.node_elems, (double2*)c.d_fac, c.dim,
-                                                         c.fac_twisted ? 1 : 0, c.d_status);
+                                                         c.fac_twisted ? tile_store(c) : TileStore{0, 1}, c.d_status);
   }
   return cudaGetLastError();
 }

@@ -6,7 +6,7 @@
 // reads them from a device table that is refreshed before each replay, with a flag that
 // leaves out the problems that are not applied (converged solves): their CTAs exit at once.
 // Requires problems with the same sweep-front geometry (line width, padded width, lines)
-// and the same kernel form (two CTAs per solve on twisted factors, or one CTA per solve),
+// and the same kernel form (twisted factors, or one CTA per solve),
 // complex64.  lsweep_solve_batch_fused runs the problems' FGMRES processes in lockstep on
 // top of it.
 #include <algorithm>
@@ -101,7 +101,7 @@ struct Fused {
     for (Ctx* c : cs) {
       if (!c->c64() || c->p.windows || c->cube || c->dim != r0.dim || c->bmax != r0.bmax ||
           c->bpmax != r0.bpmax || c->Lmax != r0.Lmax || front_form(*c) != front_form(r0) ||
-          front_form(r0) == 0) {
+          front_form(r0) == 0 || (c->twisted() && !twist_fused_fits(*c))) {
         msg = "problems need complex64 factors, no windows, no cube CDD, the same line width, "
               "padded width "
               "and line count, and the same sweep-front form (two CTAs per solve on twisted "

@@ -204,14 +204,79 @@ __device__ __host__ inline void source_lines(const SubGeom& g, int kind, int dim
   }
 }
 
+// Lines [lo, hi] of a local solution that anyone reads (2D sweeps towards rising or falling
+// y): the owned lines and the two across the face the sweep leaves by, and on the vertical
+// faces the rows of Q, the only ones the traces R_UP, L_UP, R_DOWN and L_DOWN are read at.
+// The lines on the other side of Q are not computed.  All lines for every other task.
+__device__ __host__ inline void needed_lines(const SubGeom& g, int kind, int dim, int& lo,
+                                             int& hi) {
+  const int rc = dim == 2 && kind != K_RAW ? row_cond(kind) : 0, m = (g.L - 1) / 2;
+  lo = rc == 1 ? (g.oy0 < m ? g.oy0 : m) : 0;
+  hi = rc == 2 ? (g.oy1 - 1 > m ? g.oy1 - 1 : m) : g.L - 1;
+}
+
 // Middle line of a twisted factor (lines 0..m-1 eliminated from line 0, lines L-1..m+1 from
 // line L-1, line m last): it balances the two substitution chains of a twisted solve.
 __device__ __host__ inline int twist_line(int L) { return (L - 1) / 2; }
 
-// Factor blocks one local solve streams, forward and backward: 2 L, less the forward steps
-// over zero right-hand sides that the sweep kernel skips.  form: 0 no skip (cluster-split
-// kernels), 1 one CTA per solve (forward from line 0), 2 two CTAs per solve on the twisted
-// factor (forward from both ends towards twist_line(L)).
+// Storage of a twisted factor's blocks.  The local operator is complex symmetric, so each
+// block inverse is too, and only its lower triangle is stored, in square tiles of T x T
+// entries (G = ceil(b / T) tile rows, the last one padded with zeros): one thread of the sweep
+// kernel holds one tile.  NQ CTAs share a block: tile (I, J), I > J, belongs to CTA (I + J) % NQ
+// and the triangle of diagonal tile I to CTA I % NQ.  The part of one CTA is contiguous: its
+// tiles, interleaved so that a warp reads consecutive 16-byte units (unit u of all tiles side by
+// side), its diagonal triangles, interleaved likewise by entry, and the couplings c_k and
+// c_{k-1}, each padded to an even count, so that every part starts on 16 bytes.
+struct TileStore {
+  int T, NQ;             // tile width (0: blocks stored whole), CTAs sharing a block
+};
+__device__ __host__ inline int tile_rows(int b, int T) { return (b + T - 1) / T; }
+__device__ __host__ inline int tile_count(int G, int NQ, int q) {
+  return NQ == 1 ? G * (G - 1) / 2 : q ? G * G / 4 : (G - 1) * (G - 1) / 4;
+}
+__device__ __host__ inline int diag_count(int G, int NQ, int q) {
+  return NQ == 1 ? G : q ? G / 2 : (G + 1) / 2;
+}
+// index of tile (I, J), I > J, among its CTA's
+__device__ __host__ inline int tile_number(int I, int J, int NQ) {
+  if (NQ == 1) return I * (I - 1) / 2 + J;
+  return (I + J) & 1 ? I * I / 4 + (J - ((I + 1) & 1)) / 2
+                     : (I - 1) * (I - 1) / 4 + (J - (I & 1)) / 2;
+}
+__device__ __host__ inline int part_cpl(int b, TileStore s, int q) {   // offset of the couplings
+  const int G = tile_rows(b, s.T);
+  return tile_count(G, s.NQ, q) * s.T * s.T +
+         ((diag_count(G, s.NQ, q) * (s.T * (s.T + 1) / 2) + 1) & ~1);
+}
+__device__ __host__ inline int part_elems(int b, TileStore s, int q) {
+  return part_cpl(b, s, q) + 2 * ((b + 1) & ~1);
+}
+__device__ __host__ inline int block_elems(int b, TileStore s) {
+  return part_elems(b, s, 0) + (s.NQ > 1 ? part_elems(b, s, 1) : 0);
+}
+// entry (r, c) of a block whose entries are es bytes (8 or 16)
+__device__ __host__ inline int tile_index(int b, TileStore s, int es, int r, int c) {
+  if (r < c) {
+    const int t = r;
+    r = c;
+    c = t;
+  }
+  const int T = s.T, I = r / T, J = c / T, G = tile_rows(b, T);
+  const int q = s.NQ == 1 ? 0 : (I + J) & 1;
+  if (I > J) {
+    const int P = 16 / es, e = (r - I * T) * T + c - J * T;
+    return (q ? part_elems(b, s, 0) : 0) +
+           ((e / P) * tile_count(G, s.NQ, q) + tile_number(I, J, s.NQ)) * P + e % P;
+  }
+  const int qd = s.NQ == 1 ? 0 : I & 1, d = s.NQ == 1 ? I : I >> 1, i = r - I * T, j = c - I * T;
+  return (qd ? part_elems(b, s, 0) : 0) + tile_count(G, s.NQ, qd) * T * T +
+         (i * (i + 1) / 2 + j) * diag_count(G, s.NQ, qd) + d;
+}
+
+// Factor blocks one local solve uses, forward and backward: 2 L, less the steps that the
+// sweep kernel skips.  form: 0 no skip (cluster-split kernels), 1 one CTA per solve (forward
+// from line 0; skips forward steps over zero right-hand sides), 2 twisted factors (forward
+// from both ends towards twist_line(L); also skips backward steps past needed_lines).
 __device__ __host__ inline int solve_blocks(const SubGeom& g, int kind, int dim, int form) {
   int lo, hi;
   source_lines(g, kind, dim, lo, hi);
@@ -220,7 +285,9 @@ __device__ __host__ inline int solve_blocks(const SubGeom& g, int kind, int dim,
   if (form == 2) {
     const int m = twist_line(L);
     const int s0 = lo < m ? lo : m, s1 = L - 1 - hi < L - 1 - m ? L - 1 - hi : L - 1 - m;
-    return 2 * L - s0 - s1;
+    int nlo, nhi;
+    needed_lines(g, kind, dim, nlo, nhi);
+    return 2 * L - s0 - s1 - nlo - (L - 1 - nhi);
   }
   return 2 * L;
 }
@@ -289,7 +356,6 @@ struct Ctx {
   int red_blocks = 0;
   bool factored = false;        // (a clone asks its parent: is_factored)
   bool fac_twisted = false;     // factors twisted at twist_line(L) (set by lsweep_factor)
-  int quad_cap = -1;            // four-CTA sweep clusters the device runs at once (-1: unknown)
   // a clone shares the parent's coefficients, factors and plan and owns only its working
   // buffers (lanes, traces, Krylov space, gradient workspace) and its stream
   Ctx* parent = nullptr;
@@ -333,9 +399,8 @@ struct Ctx {
   std::vector<Ctx*> shifted;
   double* d_psi = nullptr;
   double2* d_win = nullptr;
-  // line vectors of the sweep kernels that keep them in global memory (complex128 four-CTA
-  // kernel; wide kernel with clusters of 4-8 CTAs), one region per CTA of the largest level
-  // (allocated with the working buffers, lines_bytes)
+  // line vectors of the wide sweep kernel where they do not fit shared memory, one region per
+  // CTA of the largest level (allocated with the working buffers, lines_bytes)
   void* d_lines = nullptr;
   long long spin() const { return p.max_spin > 0 ? p.max_spin : (1LL << 30); }
   // complex64 factors and sweeps (every precision but LSWEEP_C128)
@@ -386,11 +451,19 @@ cudaError_t launch_sum_lanes(Ctx& c, double2* z, bool accumulate = false);
 // the CDD shifted by (a, b) half blocks
 cudaError_t launch_window_tables(Ctx& c);
 cudaError_t launch_window(Ctx& c, const double2* r, double2* out, int a, int b);
-// block sweeps over K right-hand sides (sweep_multi.cu): the geometry of the kernel (false
-// when it does not apply), whether a handle can use it, the line-vector elements per CTA,
-// and one level's launch with the lanes and traces of rhs[0..K) and the inputs r[0..K)
-bool multi_geometry(const Ctx& c, int K, int& threads, int& nslot, unsigned& slot_bytes,
-                    size_t& smem);
+// twisted kernels (twist.cu): whether they take a plan's lines (and in a fused application),
+// the local solves the device runs at once, one level's launch
+struct FrontArgs;
+bool twist_fits(const Ctx& c);
+// storage of a plan's twisted blocks
+TileStore tile_store(const Ctx& c);
+bool twist_fused_fits(const Ctx& c);
+int twist_concurrency(const Ctx& c);
+cudaError_t launch_twist(Ctx& c, const FrontArgs& a, int count, const FrontArgs* table,
+                         cudaStream_t stream);
+// block sweeps over K right-hand sides (twist.cu): whether a handle can use them, the
+// line-vector elements per CTA, and one level's launch with the lanes and traces of
+// rhs[0..K) and the inputs r[0..K)
 bool multi_supported(const Ctx& c, int K);
 long long multi_line_stride(const Ctx& c, int K);
 cudaError_t launch_front_multi(Ctx& c, int li, int K, Ctx* const* rhs, const double2* const* r);
@@ -399,12 +472,12 @@ void set_global_error(const std::string& msg);
 bool front_pipeline_fits(const Ctx& c);
 // bytes of global line-vector scratch (d_lines) the plan's sweep kernels need (0: none)
 size_t lines_bytes(const Ctx& c);
-// true when lsweep_factor should store twisted factors: complex64, sweep-front kernel 0
-// (automatic) or 3, and the two-CTA kernel fits the widest line
+// true when lsweep_factor should store twisted factors: sweep-front kernel 0 (automatic) or 3,
+// and the twisted kernels fit the widest line
 bool wants_twisted(const Ctx& c);
 // local solves the GPU runs at once with the sweep-front kernel chosen at setup (the
-// co-resident clusters of two CTAs, or CTAs, on the current device; a 152-SM GB300 when no
-// device is visible), or 0 when the plan's kernel splits solves by front size (no limit)
+// co-resident clusters, or CTAs, on the current device; a 152-SM GB300 when no device is
+// visible), or 0 when the plan's kernel splits solves by front size (no limit)
 int front_concurrency(const Ctx& c);
 cudaError_t launch_matvec(Ctx& c, const double2* x, double2* y);
 cudaError_t launch_extend_source(Ctx& c, const double* f_bulk, double2* f_ext);

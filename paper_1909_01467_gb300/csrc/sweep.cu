@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(768, 1) k_front(FrontArgs a, Pipe pp, int* sta
 // the warp by a 12-shuffle transpose.  The row's owner lane (lane 8q) updates the line
 // vectors (shared memory) and publishes the next right-hand entry; one named barrier per
 // step orders the double-buffered vector.  No global memory is touched inside the loop.
-// kFused: as for k_front_pair.
+// kFused: as for k_twist.
 template <bool kFused>
 __global__ void __launch_bounds__(768, 1) k_front_solo(FrontArgs a_, int Lmax, int bmax, int nslot,
                                                        unsigned slot_bytes, int PD,
@@ -391,552 +391,9 @@ __global__ void __launch_bounds__(768, 1) k_front_solo(FrontArgs a_, int Lmax, i
   front_epilogue<float2>(a, g, kind, sub, yl, R);
 }
 
-// ---- two CTAs per solve on a twisted factor (complex64, b <= 92) -------------------------
-//
-// A factor twisted at m = twist_line(L) holds, for the lines above m, the inverses D_k^-1 of
-// the elimination from line 0, for the lines below m the inverses E_k^-1 of the elimination
-// from line L - 1, and at m the inverse of T_m = A_mm - c_{m-1} D_{m-1}^-1 c_{m-1}
-// - c_m E_{m+1}^-1 c_m (c_k: diagonal coupling of lines k and k + 1).  The substitution then
-// splits into two chains of about L steps that meet once, run side by side by the two CTAs
-// of a cluster:
-//   CTA 0:  y_k = D_k^-1 (g_k - c_{k-1} y_{k-1}),  k = 0 .. m-1;
-//   CTA 1:  z_k = E_k^-1 (g_k - c_k z_{k+1}),      k = L-1 .. m+1;
-// each sends its part of line m's right-hand side (-c_{m-1} y_{m-1}, resp. -c_m z_{m+1}) into
-// the other's shared memory (st.async completing on the receiver's mbarrier), both form
-//   x_m = T_m^-1 (g_m - c_{m-1} y_{m-1} - c_m z_{m+1})
-// and return outwards:  x_k = y_k - D_k^-1 (c_k x_{k+1})      (k < m, CTA 0),
-//                       x_k = z_k - E_k^-1 (c_{k-1} x_{k-1})  (k > m, CTA 1).
-// A solve's dependent chain is about half that of one CTA, and a front launches twice as
-// many CTAs.  Within a CTA the step is the one-CTA kernel's (whole stored blocks through a
-// TMA ring, four rows per consumer warp, shuffle transpose-reduction, one named barrier).
-// CTA 0 writes lines 0..m of the solution, CTA 1 lines m+1..L-1.
-// kFused: one launch over the solves of several problems (fused applications): the task's
-// kind carries its problem in bits 8.., whose arguments come from `table`; a problem marked
-// skip is not applied (its CTAs exit at once).
-template <bool kFused>
-__global__ void __launch_bounds__(768, 1) k_front_pair(FrontArgs a_, int Lmax, int bmax, int nslot,
-                                                       unsigned slot_bytes, int PD,
-                                                       const FrontArgs* __restrict__ table,
-                                                       int* status) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  griddep_launch_dependents();                          // the next level may start its setup
-  const Task task = a_.tasks[a_.task_off + blockIdx.x / 2];
-  const FrontArgs& a = kFused ? table[task.kind >> 8] : a_;
-  if (kFused && a.skip) return;
-  const int sub = task.sub, kind = kFused ? (task.kind & 0xff) : task.kind;
-  const SubGeom g = a.subs[sub];
-  const int b = g.b, bp = g.bp, L = g.L;
-  const int h = (int)cluster_rank();                   // 0: from line 0; 1: from line L - 1
-  const uint32_t peer = (uint32_t)(h ^ 1);
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int ncw = (int)(blockDim.x >> 5) - 1;          // consumer warps; the last is the producer
-  const int ncons = ncw * 32;
-  const int m = twist_line(L);
-  const int nf = h ? L - 1 - m : m;                    // steps before the middle line
-  const int nsteps = 2 * nf + 1;
-  // forward steps over lines whose right-hand side is zero give exact zeros: skip them
-  int slo, shi;
-  source_lines(g, kind, a.dim, slo, shi);
-  const int f0 = h ? min(L - 1 - shi, nf) : min(slo, nf);
-  const int nit = nsteps - f0;                         // steps this CTA runs: s = f0 + it
-  Rows R;
-  R.RB = b;
-  R.r0 = 0;
-  R.r1 = b;
-  // shared memory: ring[nslot][slot_bytes] | full[8] | empty[8] | xbar[2] | vb[2][128] |
-  // xb[128] | yl[Lmax][bmax]
-  unsigned char* ring = smem_raw;
-  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)nslot * slot_bytes);
-  uint64_t* empty = full + kSoloMaxSlots;
-  uint64_t* xbar = empty + kSoloMaxSlots;              // the partner's part of line m has landed
-  uint32_t* xsent = reinterpret_cast<uint32_t*>(xbar + 1);   // this CTA sent its part of line m
-  float2* vb = reinterpret_cast<float2*>(xbar + 2);
-  float2* xb = vb + 2 * kSoloNV;                       // the partner's part of line m
-  float2* yl = xb + kSoloNV;                           // line vectors [L][b]
-  const float2* fac = reinterpret_cast<const float2*>(a.fac) + g.fac_off;
-  const uint32_t blk_bytes = (uint32_t)((size_t)g.bs * sizeof(float2));
-  auto blk = [&](int s) {
-    if (s < nf) return h ? L - 1 - s : s;
-    return h ? m + (s - nf) : m - (s - nf);
-  };
-  auto src = [&](int it) { return fac + (size_t)blk(f0 + it) * g.bs; };
-  bool timed_out = false;
-
-  if (tid == 0) {
-    for (int i = 0; i < nslot; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], (uint32_t)ncw);
-    }
-    mbar_init(xbar, 1);
-    *xsent = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    mbar_expect_tx(xbar, (uint32_t)(b * sizeof(float2)));   // one entry per row from the partner
-  }
-  for (int t = tid; t < 3 * kSoloNV; t += blockDim.x) vb[t] = make_float2(0.f, 0.f);
-  __syncthreads();
-  cluster_sync_all();                                  // the partner's xbar is armed
-  if (w == ncw && lane == 0) {
-    for (int t = 0; t < min(PD, nit); ++t) bulk_prefetch_l2(src(t), blk_bytes);
-    for (int t = 0; t < min(nslot, nit); ++t) {
-      mbar_expect_tx(&full[t], blk_bytes);
-      bulk_g2s(ring + (size_t)t * slot_bytes, src(t), blk_bytes, &full[t]);
-    }
-  }
-  griddep_wait();                                       // traces of the previous level
-  build_source<float2>(a, g, kind, yl, R);
-  __syncthreads();
-
-  if (w == ncw) {
-    // ---- producer: refill each slot once every consumer warp has released it; before the
-    // CTA may exit, wait for every copy it issued -----------------------------------------
-    if (lane == 0) {
-      int issued = min(nslot, nit);
-      for (int t = nslot; t < nit; ++t) {
-        const int slot = t % nslot;
-        mbar_wait<false>(&empty[slot], (uint32_t)((t / nslot - 1) & 1), status, timed_out, a.spin);
-        if (timed_out) break;
-        if (PD > 0 && t + PD < nit) bulk_prefetch_l2(src(t + PD), blk_bytes);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(&full[slot], blk_bytes);
-        bulk_g2s(ring + (size_t)slot * slot_bytes, src(t), blk_bytes, &full[slot]);
-        issued = t + 1;
-      }
-      drain_ring(full, nslot, issued, status);
-    }
-  } else {
-    // ---- consumers ---------------------------------------------------------------------
-    const int r0 = 4 * w;
-    const int orow = r0 + (lane >> 3);                  // row of this lane after the reduction
-    const bool owner = (lane & 7) == 0 && orow < b;
-    const uint32_t rx = mapa(smem_u32(xb + orow), peer), rbar = mapa(smem_u32(xbar), peer);
-    if (f0 < nf) {
-      if (tid < b) vb[tid] = yl[(size_t)blk(f0) * b + tid];   // first right-hand side
-    } else if (owner) {
-      // the middle line comes first: this side adds nothing to its right-hand side (no
-      // lines before it, or zero right-hand sides on all of them)
-      st_async(rx, make_float2(0.f, 0.f), rbar);
-      *(volatile uint32_t*)xsent = 1;
-      mbar_wait<true>(xbar, 0, status, timed_out, a.spin);
-      vb[orow] = yl[(size_t)m * b + orow] + xb[orow];
-    }
-    int it_end = nit;
-    if (bar_red_or(timed_out, ncons)) it_end = 0;
-    int slot = 0;
-    uint32_t phase = 0;
-    for (int it = 0; it < it_end; ++it) {
-      const int s = f0 + it;
-      const int k = blk(s);
-      mbar_wait<false>(&full[slot], phase, status, timed_out, a.spin);
-      const float2* D = reinterpret_cast<const float2*>(ring + (size_t)slot * slot_bytes);
-      const float2* Dw = D + (size_t)r0 * bp + lane;
-      const float2* v = vb + (size_t)(it & 1) * kSoloNV;
-      // the owner's operands that do not depend on this step's sums, read first.  Forward:
-      // g of the next line inwards and the coupling towards it; middle and backward: y_k
-      // (backward only) and the coupling towards the next line outwards.  Row b of a block
-      // holds c_k, row b + 1 holds c_{k-1}.
-      float2 Aval = make_float2(0.f, 0.f), cpl = Aval;
-      if (owner) {
-        if (s < nf) {
-          Aval = yl[(size_t)(h ? k - 1 : k + 1) * b + orow];
-          cpl = D[(size_t)(h ? b + 1 : b) * bp + orow];
-        } else {
-          if (s > nf) Aval = yl[(size_t)k * b + orow];
-          cpl = D[(size_t)(h ? b : b + 1) * bp + orow];
-        }
-      }
-      // unguarded reads: as in the one-CTA kernel (the slot covers 4 W rows of bp + 96)
-      float2 vr[3], vi[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float2 x = v[lane + 32 * c];
-        vr[c] = make_float2(x.x, x.x);
-        vi[c] = make_float2(x.y, x.y);
-      }
-      float re[4], im[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float2 P = make_float2(0.f, 0.f), Q = P;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float2 d = Dw[q * bp + 32 * c];
-          P = __ffma2_rn(d, vr[c], P);
-          Q = __ffma2_rn(d, vi[c], Q);
-        }
-        re[q] = P.x - Q.y;
-        im[q] = Q.x + P.y;
-      }
-      __syncwarp();
-      // this warp is done with the slot; a warp whose wait gave up never releases it (the
-      // copy may still be landing), so the producer refills no slot with a copy in flight
-      if (lane == 0 && !timed_out) mbar_arrive(&empty[slot]);
-      if (++slot == nslot) {
-        slot = 0;
-        phase ^= 1u;
-      }
-      const bool h16 = lane & 16, h8 = lane & 8;
-      float kr0 = h16 ? re[2] : re[0], ki0 = h16 ? im[2] : im[0];
-      float kr1 = h16 ? re[3] : re[1], ki1 = h16 ? im[3] : im[1];
-      const float or0 = h16 ? re[0] : re[2], oi0 = h16 ? im[0] : im[2];
-      const float or1 = h16 ? re[1] : re[3], oi1 = h16 ? im[1] : im[3];
-      kr0 += __shfl_xor_sync(0xffffffffu, or0, 16);
-      ki0 += __shfl_xor_sync(0xffffffffu, oi0, 16);
-      kr1 += __shfl_xor_sync(0xffffffffu, or1, 16);
-      ki1 += __shfl_xor_sync(0xffffffffu, oi1, 16);
-      float kr = h8 ? kr1 : kr0, ki = h8 ? ki1 : ki0;
-      const float orr = h8 ? kr0 : kr1, oii = h8 ? ki0 : ki1;
-      kr += __shfl_xor_sync(0xffffffffu, orr, 8);
-      ki += __shfl_xor_sync(0xffffffffu, oii, 8);
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        kr += __shfl_xor_sync(0xffffffffu, kr, o);
-        ki += __shfl_xor_sync(0xffffffffu, ki, o);
-      }
-      if (owner) {
-        const float2 sum = make_float2(kr, ki);
-        float2 nv = make_float2(0.f, 0.f);
-        float2* yk = yl + (size_t)k * b + orow;
-        if (s < nf) {
-          *yk = sum;                                    // y_k (z_k)
-          const float2 c = cmul(cpl, sum);
-          nv = Aval - c;
-          if (s + 1 == nf) {
-            // next is the middle line: exchange the two sides' parts of its right-hand side
-            // (every owner of this CTA sends in this step, timed out or not: all or none)
-            st_async(rx, make_float2(-c.x, -c.y), rbar);
-            *(volatile uint32_t*)xsent = 1;
-            mbar_wait<true>(xbar, 0, status, timed_out, a.spin);
-            nv = nv + xb[orow];
-          }
-        } else {
-          const float2 x = s == nf ? sum : Aval - sum;  // x_m, or x_k = y_k - D_k^-1 (c x)
-          *yk = x;
-          if (s + 1 < nsteps) nv = cmul(cpl, x);
-        }
-        vb[(size_t)((it + 1) & 1) * kSoloNV + orow] = nv;
-      }
-      if (bar_red_or(timed_out, ncons)) break;          // a wait gave up: leave together
-    }
-  }
-  const bool gave_up = __syncthreads_or(timed_out) != 0;
-  cluster_sync_all();                                   // both halves have left their loops
-  if (gave_up && tid == 0) {
-    // A CTA that did not give up has seen the partner's part of line m land.  After a
-    // timeout, if the partner sent its part (it sends all rows or none), wait (bounded)
-    // until the stores have landed in this CTA before it exits.
-    if (ld_cluster_u32(mapa(smem_u32(xsent), peer)) != 0) mbar_drain<true>(xbar, 0, status);
-  }
-  Rows Rout = R;                                        // this CTA's lines of the solution
-  Rout.k0 = h ? m + 1 : 0;
-  Rout.k1 = h ? L : m + 1;
-  front_epilogue<float2>(a, g, kind, sub, yl, Rout);
-}
-
-// ---- four CTAs per solve on a twisted factor: rows split in two (b <= 92) ----------------
-//
-// For dependency levels with few solves (the end of the diagonal sweeps' dependency chain,
-// where one solve's latency sets the level's time) each half of a twisted solve (see
-// k_front_pair) is split by rows over two CTAs: CTA (h, q) of a cluster of four (rank
-// 2 h + q) streams rows [q RB, q RB + nr) of each stored block plus the two coupling rows
-// (two bulk copies per step) and forms those rows of the block product, so each CTA reads
-// half the factor bytes per step.  After each step the row owners send the next right-hand
-// entries of their rows to the other CTA of the same half (st.async completing on its
-// mbarrier), and at the last forward step their part of the middle line's right-hand side
-// to both CTAs of the other half.  The arithmetic of every row is the two-CTA kernel's, so
-// the results are the same bit for bit.  CTA (h, q) writes rows [q RB, q RB + nr) of its
-// half's lines.
-// complex128 (the plain form): a half block of 48 rows is 75 KB, so two ring slots fit but
-// not the solve's line vectors as well; those (L x b entries per CTA) live in global memory
-// (`lines`, one region per CTA) and an owner's next line entry is loaded at the start of the
-// step, before the step's waits.  The products are FP64 FMAs.
-template <typename C>
-__global__ void __launch_bounds__(416, 1) k_front_quad(FrontArgs a, int Lmax, int bmax, int RB,
-                                                       int nslot, unsigned slot_bytes, int PD,
-                                                       C* lines, int* status) {
-  using Real = decltype(C{}.x);
-  constexpr bool kGlobalLines = std::is_same<C, double2>::value;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  griddep_launch_dependents();                          // the next level may start its setup
-  const Task task = a.tasks[a.task_off + blockIdx.x / 4];
-  const int sub = task.sub, kind = task.kind;
-  const SubGeom g = a.subs[sub];
-  const int b = g.b, bp = g.bp, L = g.L;
-  const int rank = (int)cluster_rank();
-  const int h = rank >> 1, q = rank & 1;               // half (0: from line 0), row group
-  const uint32_t mate = (uint32_t)(rank ^ 1);          // the other row group of this half
-  const uint32_t oth0 = (uint32_t)(2 * (h ^ 1)), oth1 = oth0 + 1;   // the other half
-  const int r0 = q * RB;
-  const int nr = max(0, min(b, r0 + RB) - r0);          // rows of this CTA
-  auto rows_of = [&](int qq) { return max(0, min(b, qq * RB + RB) - qq * RB); };
-  const int nr_mate = rows_of(q ^ 1);
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int ncw = (int)(blockDim.x >> 5) - 1;          // consumer warps; the last is the producer
-  const int ncons = ncw * 32;
-  const int m = twist_line(L);
-  const int nf = h ? L - 1 - m : m;
-  const int nsteps = 2 * nf + 1;
-  int slo, shi;
-  source_lines(g, kind, a.dim, slo, shi);
-  const int f0 = h ? min(L - 1 - shi, nf) : min(slo, nf);
-  const int nit = nsteps - f0;                         // steps run: s = f0 + it
-  Rows R;
-  R.RB = b;
-  R.r0 = 0;
-  R.r1 = b;
-  // shared memory: ring[nslot][slot_bytes] | full[8] | empty[8] | vbar[2] | xbar[2] |
-  // flags[4] (32-bit) | vb[2][128] | xb[128] | yl[Lmax][bmax]; a slot holds the CTA's nr rows
-  // of a block and then the two coupling rows
-  unsigned char* ring = smem_raw;
-  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)nslot * slot_bytes);
-  uint64_t* empty = full + kSoloMaxSlots;
-  uint64_t* vbar = empty + kSoloMaxSlots;              // the mate's entries of the next vector
-  uint64_t* xbar = vbar + 2;                           // xbar[qq]: the rows of line m's part
-                                                       // sent by CTA (other half, qq)
-  // flags[0]: this CTA sent its part of line m to the other half (all rows or none);
-  // flags[1]: the last step whose vector entries this CTA sent to its mate
-  uint32_t* flags = reinterpret_cast<uint32_t*>(xbar + 2);
-  C* vb = reinterpret_cast<C*>(xbar + 4);
-  C* xb = vb + 2 * kSoloNV;
-  C* yl = kGlobalLines ? lines + (size_t)blockIdx.x * Lmax * bmax : xb + kSoloNV;
-  const C* fac = reinterpret_cast<const C*>(a.fac) + g.fac_off;
-  const uint32_t slab_bytes = (uint32_t)((size_t)nr * bp * sizeof(C));
-  const uint32_t cpl_bytes = (uint32_t)((size_t)2 * bp * sizeof(C));
-  auto blk = [&](int s) {
-    if (s < nf) return h ? L - 1 - s : s;
-    return h ? m + (s - nf) : m - (s - nf);
-  };
-  auto src = [&](int it) { return fac + (size_t)blk(f0 + it) * g.bs; };
-  auto issue = [&](int it, int slot) {
-    unsigned char* dst = ring + (size_t)slot * slot_bytes;
-    const C* s0 = src(it);
-    mbar_expect_tx(&full[slot], slab_bytes + cpl_bytes);
-    if (nr > 0) bulk_g2s(dst, s0 + (size_t)r0 * bp, slab_bytes, &full[slot]);
-    bulk_g2s(dst + slab_bytes, s0 + (size_t)b * bp, cpl_bytes, &full[slot]);
-  };
-  auto vparity = [](int it) { return (uint32_t)(((it - 1) >> 1) & 1); };
-  bool timed_out = false;
-
-  if (tid == 0) {
-    for (int i = 0; i < nslot; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], (uint32_t)ncw);
-    }
-    mbar_init(&vbar[0], 1);
-    mbar_init(&vbar[1], 1);
-    mbar_init(&xbar[0], 1);
-    mbar_init(&xbar[1], 1);
-    flags[0] = flags[1] = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // the rows of the other half's two CTAs
-    mbar_expect_tx(&xbar[0], (uint32_t)(rows_of(0) * sizeof(C)));
-    mbar_expect_tx(&xbar[1], (uint32_t)(rows_of(1) * sizeof(C)));
-    if (nit > 1) mbar_expect_tx(&vbar[1], (uint32_t)(nr_mate * sizeof(C)));   // it = 1
-    if (nit > 2) mbar_expect_tx(&vbar[0], (uint32_t)(nr_mate * sizeof(C)));   // it = 2
-  }
-  for (int t = tid; t < 3 * kSoloNV; t += blockDim.x) vb[t] = czero<C>();
-  __syncthreads();
-  cluster_sync_all();                                  // every CTA's barriers are armed
-  if (w == ncw && lane == 0) {
-    for (int t = 0; t < min(PD, nit); ++t) bulk_prefetch_l2(src(t), (uint32_t)((size_t)g.bs * sizeof(C)));
-    for (int t = 0; t < min(nslot, nit); ++t) issue(t, t);
-  }
-  griddep_wait();                                       // traces of the previous level
-  build_source<C>(a, g, kind, yl, R);
-  __syncthreads();
-
-  int it_end = nit;                                   // 0 when the prologue's wait gave up
-  int varmed = nit > 2 ? 2 : nit - 1;                   // (tid 0) last step armed on vbar
-  int vok = 0;                                          // (tid 0) last step waited for
-  if (w == ncw) {
-    // ---- producer (drains every copy it issued before the CTA may exit) ----------------
-    if (lane == 0) {
-      int issued = min(nslot, nit);
-      for (int t = nslot; t < nit; ++t) {
-        const int slot = t % nslot;
-        mbar_wait<false>(&empty[slot], (uint32_t)((t / nslot - 1) & 1), status, timed_out, a.spin);
-        if (timed_out) break;
-        if (PD > 0 && t + PD < nit)
-          bulk_prefetch_l2(src(t + PD), (uint32_t)((size_t)g.bs * sizeof(C)));
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(t, slot);
-        issued = t + 1;
-      }
-      drain_ring(full, nslot, issued, status);
-    }
-  } else {
-    // ---- consumers ---------------------------------------------------------------------
-    const int lr0 = 4 * w;                              // local rows of this warp
-    const int lrow = lr0 + (lane >> 3);
-    const int orow = r0 + lrow;                         // row of this lane after the reduction
-    const bool owner = (lane & 7) == 0 && lrow < nr;
-    const uint32_t mv0 = mapa(smem_u32(vb + orow), mate);
-    const uint32_t mv1 = mapa(smem_u32(vb + kSoloNV + orow), mate);
-    const uint32_t mvb0 = mapa(smem_u32(&vbar[0]), mate), mvb1 = mapa(smem_u32(&vbar[1]), mate);
-    const uint32_t ox0 = mapa(smem_u32(xb + orow), oth0), ox1 = mapa(smem_u32(xb + orow), oth1);
-    const uint32_t oxb0 = mapa(smem_u32(&xbar[q]), oth0), oxb1 = mapa(smem_u32(&xbar[q]), oth1);
-    if (f0 < nf) {
-      if (tid < b) vb[tid] = yl[(size_t)blk(f0) * b + tid];   // first right-hand side
-    } else {
-      // the middle line comes first: this half adds nothing to its right-hand side
-      if (owner) {
-        st_async(ox0, czero<C>(), oxb0);
-        st_async(ox1, czero<C>(), oxb1);
-        *(volatile uint32_t*)&flags[0] = 1;
-      }
-      mbar_wait<true>(&xbar[0], 0, status, timed_out, a.spin);
-      mbar_wait<true>(&xbar[1], 0, status, timed_out, a.spin);
-      if (tid < b) vb[tid] = yl[(size_t)m * b + tid] + xb[tid];
-    }
-    if (bar_red_or(timed_out, ncons)) it_end = 0;
-    int slot = 0;
-    uint32_t phase = 0;
-    for (int it = 0; it < it_end; ++it) {
-      const int s = f0 + it;
-      const int k = blk(s);
-      C* vcur = vb + (size_t)(it & 1) * kSoloNV;
-      // the owner's entry of the line this step combines with: the next line's source
-      // (forward) or this line's y (backward)
-      auto line_entry = [&]() {
-        C v = czero<C>();
-        if (owner) {
-          if (s < nf) v = yl[(size_t)(h ? k - 1 : k + 1) * b + orow];
-          else if (s > nf) v = yl[(size_t)k * b + orow];
-        }
-        return v;
-      };
-      C Aval = czero<C>();
-      if constexpr (kGlobalLines) Aval = line_entry();
-      if (it > 0) {
-        // the mate's rows of this step's vector; then re-arm the barrier for step it + 2
-        mbar_wait<true>(&vbar[it & 1], vparity(it), status, timed_out, a.spin);
-        consumer_sync(ncons);
-        // re-arm only after the wait succeeded: a barrier has at most one armed phase, and
-        // the mate sends step it + 2 only after it received this CTA's step it + 1, so
-        // nothing is sent to a phase that is not armed
-        if (tid == 0 && !timed_out) {
-          vok = it;
-          if (it + 2 < nit) {
-            mbar_expect_tx(&vbar[it & 1], (uint32_t)(nr_mate * sizeof(C)));
-            varmed = it + 2;
-          }
-        }
-        if (s == nf) {
-          // middle line: add the other half's part of its right-hand side
-          mbar_wait<true>(&xbar[0], 0, status, timed_out, a.spin);
-          mbar_wait<true>(&xbar[1], 0, status, timed_out, a.spin);
-          if (tid < b) vcur[tid] = vcur[tid] + xb[tid];
-          consumer_sync(ncons);
-        }
-      }
-      mbar_wait<false>(&full[slot], phase, status, timed_out, a.spin);
-      const C* D = reinterpret_cast<const C*>(ring + (size_t)slot * slot_bytes);
-      const C* Dw = D + (size_t)lr0 * bp + lane;
-      const C* C2 = D + (size_t)nr * bp;                // coupling rows b, b + 1
-      if constexpr (!kGlobalLines) Aval = line_entry();
-      C cpl = czero<C>();
-      if (owner) cpl = C2[(size_t)((s < nf) == (h != 0) ? 1 : 0) * bp + orow];
-      // unguarded reads: a warp's rows stay inside the slot (rows beyond nr are discarded;
-      // a row's columns past bp run into the next copied row or the coupling rows)
-      C vr[3], vi[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const C x = vcur[lane + 32 * c];
-        vr[c] = mk(x.x, x.x);
-        vi[c] = mk(x.y, x.y);
-      }
-      Real re[4], im[4];
-#pragma unroll
-      for (int qq = 0; qq < 4; ++qq) {
-        C P = czero<C>(), Q = P;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const C d = Dw[qq * bp + 32 * c];
-          P = fma_pair(d, vr[c], P);
-          Q = fma_pair(d, vi[c], Q);
-        }
-        re[qq] = P.x - Q.y;
-        im[qq] = Q.x + P.y;
-      }
-      __syncwarp();
-      if (lane == 0 && !timed_out) mbar_arrive(&empty[slot]);   // see k_front_solo
-      if (++slot == nslot) {
-        slot = 0;
-        phase ^= 1u;
-      }
-      const bool h16 = lane & 16, h8 = lane & 8;
-      Real kr0 = h16 ? re[2] : re[0], ki0 = h16 ? im[2] : im[0];
-      Real kr1 = h16 ? re[3] : re[1], ki1 = h16 ? im[3] : im[1];
-      const Real or0 = h16 ? re[0] : re[2], oi0 = h16 ? im[0] : im[2];
-      const Real or1 = h16 ? re[1] : re[3], oi1 = h16 ? im[1] : im[3];
-      kr0 += __shfl_xor_sync(0xffffffffu, or0, 16);
-      ki0 += __shfl_xor_sync(0xffffffffu, oi0, 16);
-      kr1 += __shfl_xor_sync(0xffffffffu, or1, 16);
-      ki1 += __shfl_xor_sync(0xffffffffu, oi1, 16);
-      Real kr = h8 ? kr1 : kr0, ki = h8 ? ki1 : ki0;
-      const Real orr = h8 ? kr0 : kr1, oii = h8 ? ki0 : ki1;
-      kr += __shfl_xor_sync(0xffffffffu, orr, 8);
-      ki += __shfl_xor_sync(0xffffffffu, oii, 8);
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) {
-        kr += __shfl_xor_sync(0xffffffffu, kr, o);
-        ki += __shfl_xor_sync(0xffffffffu, ki, o);
-      }
-      C nv = czero<C>();
-      if (owner) {
-        const C sum = mk(kr, ki);
-        C* yk = yl + (size_t)k * b + orow;
-        if (s < nf) {
-          *yk = sum;
-          const C cc = cmul(cpl, sum);
-          nv = Aval - cc;
-          if (s + 1 == nf) {
-            // every owner of this CTA sends in this step, timed out or not: all rows or none
-            const C wv = mk(-cc.x, -cc.y);
-            st_async(ox0, wv, oxb0);
-            st_async(ox1, wv, oxb1);
-            *(volatile uint32_t*)&flags[0] = 1;
-          }
-        } else {
-          const C x = s == nf ? sum : Aval - sum;
-          *yk = x;
-          if (s + 1 < nsteps) nv = cmul(cpl, x);
-        }
-        if (it + 1 < nit) vb[(size_t)((it + 1) & 1) * kSoloNV + orow] = nv;
-      }
-      if (bar_red_or(timed_out, ncons)) break;          // a wait gave up: leave together
-      // the next vector's entries go to the mate only when no wait of this CTA gave up
-      if (it + 1 < nit) {
-        const int nb = (it + 1) & 1;
-        if (owner) st_async(nb ? mv1 : mv0, nv, nb ? mvb1 : mvb0);
-        if (tid == 0) *(volatile uint32_t*)&flags[1] = (uint32_t)(it + 1);
-      }
-    }
-  }
-  const bool gave_up = __syncthreads_or(timed_out) != 0;
-  cluster_sync_all();                                   // every CTA has left its loop
-  if (gave_up && tid == 0) {
-    // Stores from the other CTAs may still be in flight.  The mate's vector entries: the
-    // steps after the last one this CTA waited for, up to the last one the mate sent (never
-    // beyond the last one armed here).  The other half's parts of line m: each of its CTAs
-    // sent all its rows or none.  Wait (bounded) until what was sent has landed.
-    const int msent = (int)ld_cluster_u32(mapa(smem_u32(&flags[1]), mate));
-    for (int t = vok + 1; t <= min(msent, varmed); ++t)
-      mbar_drain<true>(&vbar[t & 1], vparity(t), status);
-    if (ld_cluster_u32(mapa(smem_u32(&flags[0]), oth0)) != 0) mbar_drain<true>(&xbar[0], 0, status);
-    if (ld_cluster_u32(mapa(smem_u32(&flags[0]), oth1)) != 0) mbar_drain<true>(&xbar[1], 0, status);
-  }
-  Rows Rout;
-  Rout.RB = b;
-  Rout.r0 = r0;
-  Rout.r1 = r0 + nr;
-  Rout.k0 = h ? m + 1 : 0;
-  Rout.k1 = h ? L : m + 1;
-  front_epilogue<C>(a, g, kind, sub, yl + r0, Rout);   // yl + r0: rows [r0, r1) of [L][b]
-}
-
 // Geometry of the one-CTA-per-solve kernel: ring slots of one stored block, as many as fit
 // beside the line vectors (at least 2, at most kSoloMaxSlots).  False when it does not apply.
-// `extra` bytes of fixed shared memory are added after the barriers (the two-CTA kernel's
-// exchange barrier and buffer).
+// `extra` bytes of fixed shared memory are added.
 static bool solo_geometry(const Ctx& c, size_t extra, int& threads, int& nslot,
                           unsigned& slot_bytes, size_t& smem) {
   if (!c.c64() || c.bmax > 92 || c.cube) return false;   // cube plans: k_front / k_front_wide
@@ -960,63 +417,6 @@ static bool choose_solo(const Ctx& c, int& threads, int& nslot, unsigned& slot_b
                         size_t& smem) {
   return solo_geometry(c, 0, threads, nslot, slot_bytes, smem);
 }
-// the four-CTA kernel: rows per CTA RB (a multiple of 4, about b / 2), a slot of RB rows
-// plus the two coupling rows (covering the unguarded reads of 4 RB / 4 rows, columns < 96);
-// complex64 keeps the line vectors in shared memory, complex128 in global memory
-template <typename C>
-static bool choose_quad(const Ctx& c, int& threads, int& RB, int& nslot, unsigned& slot_bytes,
-                        size_t& smem) {
-  constexpr bool c64 = std::is_same<C, float2>::value;
-  if (c.c64() != c64 || c.bmax > 92 || c.cube) return false;
-  RB = ((c.bmax + 1) / 2 + 3) / 4 * 4;
-  threads = (RB / 4 + 1) * 32;
-  const size_t slot_elems = std::max((size_t)(RB + 2) * c.bpmax, (size_t)(RB - 1) * c.bpmax + 96);
-  slot_bytes = (unsigned)((slot_elems * sizeof(C) + 127) / 128 * 128);
-  const size_t fixed = (2 * kSoloMaxSlots + 6) * sizeof(uint64_t) + 3 * kSoloNV * sizeof(C) +
-                       (c64 ? (size_t)c.Lmax * c.bmax * sizeof(C) : 0);
-  const size_t limit = 227 * 1024;
-  if (fixed + 2 * (size_t)slot_bytes > limit) return false;
-  nslot = (int)std::min<size_t>(kSoloMaxSlots, (limit - fixed) / slot_bytes);
-  smem = (size_t)nslot * slot_bytes + fixed;
-  return threads <= 416;
-}
-
-// clusters of four k_front_quad CTAs the device runs at once (0 if none), computed once
-template <typename C>
-static int quad_capacity(Ctx& c) {
-  if (c.quad_cap >= 0) return c.quad_cap;
-  int th, RB, nslot;
-  unsigned slot;
-  size_t smem;
-  int ncl = 0;
-  if (choose_quad<C>(c, th, RB, nslot, slot, smem) &&
-      cudaFuncSetAttribute(k_front_quad<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(4 * 64);
-    cfg.blockDim = dim3((unsigned)th);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 4;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&ncl, k_front_quad<C>, &cfg) != cudaSuccess) ncl = 0;
-  }
-  cudaGetLastError();
-  c.quad_cap = ncl;
-  return ncl;
-}
-
-// the two-CTA kernel: also an exchange barrier (two words) and a 128-entry exchange buffer
-static bool choose_pair(const Ctx& c, int& threads, int& nslot, unsigned& slot_bytes,
-                        size_t& smem) {
-  return solo_geometry(c, 2 * sizeof(uint64_t) + kSoloNV * sizeof(float2), threads, nslot,
-                       slot_bytes, smem);
-}
-
 // ---- planes too wide for a row slab per slot: a cluster streaming chunks of rows ---------
 //
 // For 3D beams (b = Lx Ly up to ~1000 nodes per plane) one block is several MB.  A solve runs
@@ -1366,36 +766,6 @@ static bool choose_pipe(const Ctx& c, int tasks, Pipe& pp, int& threads, size_t&
   return threads <= 768 && cc <= kMaxCC && nc <= kMaxNC;
 }
 
-// A front of `count` solves on k_front_quad (twisted factors); cudaErrorNotSupported when
-// its geometry does not fit.
-template <typename C>
-static cudaError_t launch_quad(Ctx& c, const FrontArgs& a, int count, C* lines) {
-  int th, RB, nslot;
-  unsigned slot_bytes;
-  size_t smem;
-  if (!choose_quad<C>(c, th, RB, nslot, slot_bytes, smem)) return cudaErrorNotSupported;
-  const int PD = c.p.prefetch_steps < 0 ? 0 : c.p.prefetch_steps;
-  cudaError_t e = cudaFuncSetAttribute(k_front_quad<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(4 * count));
-  cfg.blockDim = dim3((unsigned)th);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = c.stream;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 4;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = c.p.pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, k_front_quad<C>, a, c.Lmax, c.bmax, RB, nslot, slot_bytes, PD,
-                            lines, c.d_status);
-}
-
 template <typename C>
 static cudaError_t launch_front_t(Ctx& c, const Task* tasks, int off, int count,
                                   const double2* rin, const double2* g_raw, double2* x_raw) {
@@ -1421,39 +791,11 @@ static cudaError_t launch_front_t(Ctx& c, const Task* tasks, int off, int count,
   a.x_raw = x_raw;
   a.spin = c.spin();
   a.skip = 0;
+  if (c.twisted()) return launch_twist(c, a, count, nullptr, c.stream);
   if constexpr (std::is_same<C, float2>::value) {
     int th, nslot;
     unsigned slot_bytes;
     size_t smem;
-    if (c.twisted()) {
-      if (c.p.front_kernel == 0 && count <= quad_capacity<float2>(c)) {
-        // a level of few solves: four CTAs per solve (rows of each half split in two)
-        cudaError_t e = launch_quad<float2>(c, a, count, nullptr);
-        if (e != cudaErrorNotSupported) return e;
-      }
-      // twisted factors: otherwise the two-CTA kernel
-      if (!choose_pair(c, th, nslot, slot_bytes, smem)) return cudaErrorInvalidConfiguration;
-      const int PD = c.p.prefetch_steps < 0 ? 0 : c.p.prefetch_steps;
-      cudaError_t e = cudaFuncSetAttribute(k_front_pair<false>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(2 * count));
-      cfg.blockDim = dim3((unsigned)th);
-      cfg.dynamicSmemBytes = smem;
-      cfg.stream = c.stream;
-      cudaLaunchAttribute at[2];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 2;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      at[1].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = c.p.pdl ? 2 : 1;
-      return cudaLaunchKernelEx(&cfg, k_front_pair<false>, a, c.Lmax, c.bmax, nslot, slot_bytes,
-                                PD, (const FrontArgs*)nullptr, c.d_status);
-    }
     if (c.p.front_kernel == 3) return cudaErrorInvalidConfiguration;   // not factored twisted
     if (c.p.front_kernel != 1 && choose_solo(c, th, nslot, slot_bytes, smem)) {
       const int PD = c.p.prefetch_steps < 0 ? 0 : c.p.prefetch_steps;
@@ -1479,10 +821,6 @@ static cudaError_t launch_front_t(Ctx& c, const Task* tasks, int off, int count,
     }
     if (c.p.front_kernel == 2) return cudaErrorInvalidConfiguration;
   }
-  if constexpr (std::is_same<C, double2>::value) {
-    // complex128 on a twisted factor: four CTAs per solve, line vectors in global memory
-    if (c.twisted()) return launch_quad<double2>(c, a, count, reinterpret_cast<double2*>(c.d_lines));
-  }
   Pipe pp;
   int th = 0;
   size_t smem = 0;
@@ -1506,41 +844,39 @@ static cudaError_t launch_front_t(Ctx& c, const Task* tasks, int off, int count,
   return cudaLaunchKernelEx(&cfg, kern, a, pp, c.d_status);
 }
 
-// One level of a fused application over several problems (k_front_pair<true> on twisted
-// factors, k_front_solo<true> on plain ones): `count` tasks from tasks[off..], each naming
-// its problem (kind >> 8) in `table`; the geometry is c's, which every problem shares.
+// One level of a fused application over several problems (k_twist on twisted factors,
+// k_front_solo on plain ones): `count` tasks from tasks[off..], each naming its problem
+// (kind >> 8) in `table`; the geometry is c's, which every problem shares.
 cudaError_t launch_front_fused(Ctx& c, const Task* tasks, int off, int count,
                                const FrontArgs* table, cudaStream_t stream) {
   FrontArgs a{};
   a.tasks = tasks;
   a.task_off = off;
+  if (c.twisted()) return launch_twist(c, a, count, table, stream);
   int th, nslot;
   unsigned slot_bytes;
   size_t smem;
-  const bool pair = c.twisted();
-  if (pair ? !choose_pair(c, th, nslot, slot_bytes, smem)
-           : !choose_solo(c, th, nslot, slot_bytes, smem))
-    return cudaErrorInvalidConfiguration;
+  if (!choose_solo(c, th, nslot, slot_bytes, smem)) return cudaErrorInvalidConfiguration;
   const int PD = c.p.prefetch_steps < 0 ? 0 : c.p.prefetch_steps;
-  auto kern = pair ? k_front_pair<true> : k_front_solo<true>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_front_solo<true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((pair ? 2 : 1) * count));
+  cfg.gridDim = dim3((unsigned)count);
   cfg.blockDim = dim3((unsigned)th);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = pair ? 2 : 1;
+  at[0].val.clusterDim.x = 1;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = c.p.pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, kern, a, c.Lmax, c.bmax, nslot, slot_bytes, PD, table,
-                            c.d_status);
+  return cudaLaunchKernelEx(&cfg, k_front_solo<true>, a, c.Lmax, c.bmax, nslot, slot_bytes, PD,
+                            table, c.d_status);
 }
 
 // clusters of k_front_wide the device runs at once (0 if it does not apply): a dependency
@@ -1576,14 +912,12 @@ static int wide_capacity(const Ctx& c) {
   return ncl;
 }
 
-// bytes of line-vector scratch the plan's sweep kernels need in global memory (d_lines):
-// the complex128 four-CTA kernel (4 CTAs per solve, Lmax x bmax each) and the wide kernel
-// with global line vectors (NS CTAs per solve, Lmax x RB each), for the largest level
+// bytes of line-vector scratch the plan's sweep kernels need in global memory (d_lines): the
+// wide kernel with global line vectors (NS CTAs per solve, Lmax x RB each), for the largest
+// level
 size_t lines_bytes(const Ctx& c) {
   size_t need = 0;
   const size_t tasks = (size_t)std::max(1, c.max_tasks);
-  if (!c.c64() && wants_twisted(c))
-    need = std::max(need, 4 * tasks * c.Lmax * c.bmax * sizeof(double2));
   Pipe pp;
   int th = 0;
   size_t smem = 0;
@@ -1605,7 +939,7 @@ bool front_pipeline_fits(const Ctx& c) {
   size_t smem;
   Wide wp;
   if (c.p.front_kernel == 2) return choose_solo(c, th, nslot, slot, smem);
-  if (c.p.front_kernel == 3) return choose_pair(c, th, nslot, slot, smem) && factor_fits_smem(c);
+  if (c.p.front_kernel == 3) return wants_twisted(c);
   if (c.c64())
     return choose_solo(c, th, nslot, slot, smem) || choose_pipe<float2>(c, 1, pp, th, smem) ||
            choose_wide<float2>(c, wp, smem);
@@ -1613,14 +947,13 @@ bool front_pipeline_fits(const Ctx& c) {
 }
 
 bool wants_twisted(const Ctx& c) {
-  int th, nslot, RB;
+  if (!factor_fits_smem(c) || !twist_fits(c)) return false;
+  if (c.p.front_kernel == 0) return true;
+  // front_kernel 3 asked for by name: the plans whose whole line vectors fit shared memory
+  int th, nslot;
   unsigned slot;
   size_t smem;
-  if (!c.c64())   // complex128: the four-CTA kernel with line vectors in global memory
-    return c.p.front_kernel == 0 && factor_fits_smem(c) &&
-           choose_quad<double2>(c, th, RB, nslot, slot, smem);
-  return (c.p.front_kernel == 0 || c.p.front_kernel == 3) &&
-         factor_fits_smem(c) && choose_pair(c, th, nslot, slot, smem);
+  return c.p.front_kernel == 3 && solo_geometry(c, 1040, th, nslot, slot, smem);
 }
 
 int front_form(const Ctx& c) {
@@ -1638,69 +971,18 @@ int front_concurrency(const Ctx& c) {
   int th, nslot;
   unsigned slot;
   size_t smem;
-  if (!c.c64()) {
-    // complex128 on twisted factors: clusters of four k_front_quad CTAs
-    int RB = 0, dev = 0, sms = 0, ncl = 0;
-    if (!wants_twisted(c) || !choose_quad<double2>(c, th, RB, nslot, slot, smem))
-      return c.dim == 3 ? wide_capacity<double2>(c) : 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        sms < 1) {
-      cudaGetLastError();
-      return 152 / 4;
-    }
-    if (cudaFuncSetAttribute(k_front_quad<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) == cudaSuccess) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(4 * sms));
-      cfg.blockDim = dim3((unsigned)th);
-      cfg.dynamicSmemBytes = smem;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 4;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&ncl, k_front_quad<double2>, &cfg) != cudaSuccess) ncl = 0;
-    }
-    cudaGetLastError();
-    return ncl > 0 ? ncl : sms / 4;
-  }
-  const bool pair = wants_twisted(c) && choose_pair(c, th, nslot, slot, smem);
-  const bool solo = !pair && c.p.front_kernel != 1 && choose_solo(c, th, nslot, slot, smem);
-  if (!pair && !solo) {
-    // planes too wide for a row slab (3D beams): levels of at most the co-resident clusters
-    // fill whole waves; other cluster-split plans take no limit
+  if (wants_twisted(c)) return twist_concurrency(c);
+  // planes too wide for a row slab (3D beams): levels of at most the co-resident clusters
+  // fill whole waves; other cluster-split plans take no limit
+  if (!c.c64()) return c.dim == 3 ? wide_capacity<double2>(c) : 0;
+  if (c.p.front_kernel == 1 || !choose_solo(c, th, nslot, slot, smem))
     return c.dim == 3 ? wide_capacity<float2>(c) : 0;
-  }
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, nb = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
     cudaGetLastError();
-    return pair ? 152 / 2 : 152;
+    return 152;
   }
-  if (pair) {
-    int ncl = 0;
-    if (cudaFuncSetAttribute(k_front_pair<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) == cudaSuccess) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)(2 * sms));
-      cfg.blockDim = dim3((unsigned)th);
-      cfg.dynamicSmemBytes = smem;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = 2;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&ncl, k_front_pair<false>, &cfg) != cudaSuccess) ncl = 0;
-    }
-    cudaGetLastError();
-    return ncl > 0 ? ncl : sms / 2;
-  }
-  int nb = 0;
   if (cudaFuncSetAttribute(k_front_solo<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_front_solo<false>, th, smem) != cudaSuccess)
