@@ -91,7 +91,7 @@ void free_all(Ctx* c) {
   // buffers a clone shares with its parent
   if (!c->parent) {
     void* shared[] = {c->d_m_ext, c->d_m_bulk, c->d_alpha, c->d_gcoef, c->d_lcoef, c->d_fac,
-                      c->d_subs, c->d_tasks, c->d_segs};
+                      c->d_subs, c->d_wsubs, c->d_tasks, c->d_segs};
     for (void* p : shared)
       if (p) c->mem.put(p);
   }
@@ -442,6 +442,16 @@ int build_plan(Ctx* c) {
       c->subs.push_back(g);
     }
   }
+  // plans whose sweeps stream half rows store those
+  c->half_rows = lsw::uses_wide(*c);
+  if (c->half_rows) {
+    fac = 0;
+    for (auto& g : c->subs) {
+      g.bs = lsw::half_stride(g.b);
+      g.fac_off = fac;
+      fac += (long long)g.L * g.bs;
+    }
+  }
   c->fac_elems = fac;
   c->node_elems = node;
   // task lists of one application (Alg. computeScenario3), one launch per front
@@ -514,13 +524,13 @@ int build_plan(Ctx* c) {
         nblk[f][at] = std::max(nblk[f][at], lsw::solve_blocks(g, x.kind, c->dim, f));
     }
     // per_apply counts whole b x b blocks; the bytes of a launch are those of the storage the
-    // kernel streams (twisted factors: the triangle)
+    // kernel streams (twisted factors and half rows: the triangle)
     for (int f = 0; f < 3; ++f) {
       long long le = 0, st = 0;
       for (size_t u = 0; u < seen.size(); ++u) {
         const auto& g = c->subs[seen[u]];
         le += (long long)nblk[f][u] * g.b * (long long)g.b;
-        st += (long long)nblk[f][u] * (f == 2 ? g.b * (g.b + 1LL) / 2 : g.b * (long long)g.b);
+        st += (long long)nblk[f][u] * (f == 2 || c->half_rows ? g.b * (g.b + 1LL) / 2 : g.b * (long long)g.b);
       }
       c->per_apply_elems_f[f] += le;
       c->launch_bytes_f[f].push_back((double)st * c->welem());
@@ -630,7 +640,9 @@ int alloc_all(Ctx* c) {
             dalloc(c, &c->d_fac, (size_t)c->fac_elems * we + lsw::kFacSlackBytes) &&
             dalloc(c, &c->d_subs, c->subs.size() * sizeof(lsw::SubGeom)) &&
             dalloc(c, &c->d_tasks, c->tasks.size() * sizeof(lsw::Task)) &&
-            dalloc(c, &c->d_segs, c->segs.size() * sizeof(lsw::AlphaSeg)) && alloc_work(c);
+            dalloc(c, &c->d_segs, c->segs.size() * sizeof(lsw::AlphaSeg)) &&
+            (!c->half_rows || dalloc(c, &c->d_wsubs, c->subs.size() * sizeof(lsw::SubGeom))) &&
+            alloc_work(c);
   if (!ok) {
     cudaGetLastError();
     return fail(c, LSWEEP_ENOMEM, "device or pinned host allocation failed");
@@ -826,6 +838,16 @@ int setup_one(const lsweep_params* p, const double* m_bulk, Ctx** out, int sx, i
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(c->d_segs, c->segs.data(), c->segs.size() * sizeof(lsw::AlphaSeg),
                           cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess && c->half_rows) {
+      // (a copy from pageable memory has left the vector when the call returns)
+      std::vector<lsw::SubGeom> ws = c->subs;
+      for (size_t i = 0; i < ws.size(); ++i) {
+        ws[i].fac_off = (long long)i * c->bmax * c->bpmax;
+        ws[i].bs = 0;
+      }
+      e = cudaMemcpyAsync(c->d_wsubs, ws.data(), ws.size() * sizeof(lsw::SubGeom),
+                          cudaMemcpyHostToDevice, c->stream);
+    }
     if (e != cudaSuccess) rc = fail(c, LSWEEP_ECUDA, cudaGetErrorString(e));
   }
   if (!rc) rc = compute_coefficients(c, m_bulk, false);
@@ -1091,6 +1113,7 @@ int lsweep_clone(lsweep_handle h, void* stream, lsweep_handle* out) {
   c->alpha_entries = p->alpha_entries; c->Lmax = p->Lmax; c->bmax = p->bmax;
   c->bpmax = p->bpmax; c->trace_W = p->trace_W; c->fac_elems = p->fac_elems;
   c->pz = p->pz; c->cube = p->cube; c->n_trace_arr = p->n_trace_arr;
+  c->half_rows = p->half_rows;
   c->node_elems = p->node_elems;
   for (int f = 0; f < 3; ++f) {
     c->per_apply_elems_f[f] = p->per_apply_elems_f[f];
@@ -1326,6 +1349,12 @@ std::vector<TuneCand> tune_candidates(Ctx* c) {
   c->p.front_kernel = 1;
   c->p.prefetch_steps = -1;
   if (lsw::front_pipeline_fits(*c) && (c->clones == 0 || !tw0)) cands.push_back({1, -1});
+  // the storage laid out at setup (half rows or whole blocks) stays
+  cands.erase(std::remove_if(cands.begin(), cands.end(), [&](const TuneCand& x) {
+                c->p.front_kernel = x.kernel;
+                return lsw::uses_wide(*c) != c->half_rows;
+              }),
+              cands.end());
   c->p = saved;
   std::stable_partition(cands.begin(), cands.end(), [&](const TuneCand& x) {
     return (x.kernel == 3 || x.kernel == 0) == tw0;

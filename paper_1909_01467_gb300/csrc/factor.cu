@@ -176,6 +176,92 @@ __global__ void k_plane_schur(const SubGeom* __restrict__ subs, const C* __restr
   }
 }
 
+// Half rows: between two planes the inverse of plane k in the workspace (subs: offsets without
+// a stride per line) is stored as half rows of its symmetric part in fac (dst: the plan's
+// geometry) and replaced by the Schur complement of plane k + 1 formed from that part,
+//   A_{k+1,k+1} - diag(l_k) D_k^-1 diag(l_k)   (k = -1: the first plane).
+// One CTA of 256 threads per pair of mirrored 32 x 32 tiles (tile row blockIdx.y >= tile
+// column blockIdx.x), so that both entries of a pair are read before either is written.
+template <typename C>
+__global__ void __launch_bounds__(256) k_plane_half(const SubGeom* __restrict__ subs,
+                                                    const SubGeom* __restrict__ dst,
+                                                    const C* __restrict__ lcoef, long long cstride,
+                                                    C* __restrict__ W, C* __restrict__ fac, int dim,
+                                                    int k) {
+  __shared__ C lo[32][33], up[32][33];
+  if (blockIdx.x > blockIdx.y) return;
+  const SubGeom g = subs[blockIdx.z];
+  const int b = g.b, bp = g.bp, L = g.L, Lx = g.Lx;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  if (k >= L || r0 >= b) return;
+  const C* d = lcoef + g.node_off;
+  const C* cx = d + cstride;
+  const C* cy = d + 2 * cstride;
+  const C* cl = dim == 3 ? d + 3 * cstride : cy;
+  C* M = W + g.fac_off;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const SubGeom gd = dst[blockIdx.z];
+  C* S = fac + gd.fac_off + (long long)k * gd.bs;
+  if (k >= 0) {
+    for (int i = ty; i < 32; i += 8) {
+      const int r = r0 + i, c = c0 + tx;                  // lower tile, and its mirror image
+      lo[i][tx] = r < b && c < b ? M[(long long)r * bp + c] : czero<C>();
+      const int r2 = c0 + i, c2 = r0 + tx;
+      up[i][tx] = r2 < b && c2 < b ? M[(long long)r2 * bp + c2] : czero<C>();
+    }
+    __syncthreads();
+    const int hw = b / 2, hp = half_row(b);
+    for (int i = ty; i < 32; i += 8) {
+      // entry (r, c) of the lower tile, read along its row, and (r2, c2) of the upper one
+      const int r = r0 + i, c = c0 + tx, r2 = c0 + i, c2 = r0 + tx;
+      if (r < b && c < b) {
+        const C u = lo[i][tx], t = up[tx][i];
+        const int j = c >= r ? c - r : c - r + b;
+        const bool twice = 2 * j == b && r >= hw;         // (its pair is in row r - b / 2)
+        if (j <= hw)
+          S[(long long)r * hp + j] = twice ? czero<C>() : mk((u.x + t.x) / 2, (u.y + t.y) / 2);
+      }
+      if (r2 < b && c2 < b && r0 != c0) {
+        const C u = lo[tx][i], t = up[i][tx];
+        const int j = c2 - r2;
+        if (j <= hw) S[(long long)r2 * hp + j] = mk((u.x + t.x) / 2, (u.y + t.y) / 2);
+      }
+    }
+    if (c0 == 0) {
+      // couplings c_k and c_{k-1} of this tile row's nodes
+      const int bs = (b + 1) & ~1;
+      for (int t = threadIdx.x; t < 64; t += 256) {
+        const int p = r0 + (t & 31), kk = k - (t >> 5);
+        if (p < b) S[half_cpl(b) + (t >> 5) * bs + p] = kk >= 0 ? cl[(long long)kk * b + p] : czero<C>();
+      }
+    }
+  }
+  if (k + 1 >= L) return;
+  const long long kb = (long long)(k + 1) * b;
+  auto entry = [&](int r, int c, C s) -> C {
+    const int lw = min(r, c), df = abs(r - c);
+    C v = czero<C>();
+    if (df == 0) v = d[kb + r];
+    else if (df == 1) v = cx[kb + lw];
+    else if (dim == 3 && df == Lx) v = cy[kb + lw];
+    if (k >= 0) v = v - cmul(cmul(cl[kb - b + r], s), cl[kb - b + c]);
+    return v;
+  };
+  for (int i = ty; i < 32; i += 8) {
+    const int r = r0 + i, c = c0 + tx, r2 = c0 + i, c2 = r0 + tx;
+    if (r < b && c < b) {
+      C s = czero<C>();
+      if (k >= 0) s = mk((lo[i][tx].x + up[tx][i].x) / 2, (lo[i][tx].y + up[tx][i].y) / 2);
+      M[(long long)r * bp + c] = entry(r, c, s);
+    }
+    if (r2 < b && c2 < b && r0 != c0) {
+      C s = czero<C>();
+      if (k >= 0) s = mk((lo[tx][i].x + up[i][tx].x) / 2, (lo[tx][i].y + up[i][tx].y) / 2);
+      M[(long long)r2 * bp + c2] = entry(r2, c2, s);
+    }
+  }
+}
+
 // A_JJ <- A_JJ^-1 (one CTA per subdomain)
 template <typename C>
 __global__ void k_gj_panel(const SubGeom* __restrict__ subs, C* __restrict__ fac, int k, int j0,
@@ -316,10 +402,30 @@ __global__ void k_gj_cols(const SubGeom* __restrict__ subs, C* __restrict__ fac,
 template <typename C>
 static cudaError_t launch_factor_wide(Ctx& c) {
   const int nsub = (int)c.subs.size();
-  C* fac = reinterpret_cast<C*>(c.d_fac);
   const C* lc = reinterpret_cast<const C*>(c.d_lcoef);
   const long long bs_max = (long long)(c.bmax + 2) * c.bpmax;
   const dim3 gs((unsigned)std::min<long long>(1024, (bs_max + 255) / 256), (unsigned)nsub);
+  // whole blocks are inverted where they are stored; half rows are made from one whole block
+  // per subdomain in a workspace, which every plane passes through
+  void* W = nullptr;
+  c.f_subs = c.half_rows ? c.d_wsubs : c.d_subs;
+  c.f_fac = c.d_fac;
+  if (c.half_rows) {
+    W = c.mem.get((size_t)nsub * c.bmax * c.bpmax * sizeof(C));
+    if (!W) return cudaErrorMemoryAllocation;
+    c.f_fac = W;
+  }
+  C* fac = reinterpret_cast<C*>(c.f_fac);
+  const SubGeom* subs = c.f_subs;
+  const unsigned t32 = (unsigned)((c.bmax + 31) / 32);
+  // the Schur complement of plane k (half rows: plane k - 1 is stored on the way)
+  auto next_plane = [&](int k) {
+    if (c.half_rows)
+      k_plane_half<C><<<dim3(t32, t32, (unsigned)nsub), 256, 0, c.stream>>>(
+          subs, c.d_subs, lc, c.node_elems, fac, reinterpret_cast<C*>(c.d_fac), c.dim, k - 1);
+    else
+      k_plane_schur<C><<<gs, 256, 0, c.stream>>>(subs, lc, c.node_elems, fac, c.dim, k);
+  };
   // complex64: 128-column panels with the products on the tensor cores (three TF32 terms
   // per operand: FP32-level; one for LSWEEP_C64_TF32; three BF16 terms for
   // LSWEEP_C64_BF16X3); complex128: 32-column panels on the CUDA cores in FP64
@@ -362,7 +468,7 @@ static cudaError_t launch_factor_wide(Ctx& c) {
                                          (long long)lb, (long long)rb, prec, c.stream);
     };
     for (int k = 0; e == cudaSuccess && k < c.Lmax; ++k) {
-      k_plane_schur<C><<<gs, 256, 0, c.stream>>>(c.d_subs, lc, c.node_elems, fac, c.dim, k);
+      next_plane(k);
       e = launch_gj_panel_inverse(c, k, 0, c.stream);
       for (int j = 0; e == cudaSuccess && j < npan; ++j) {
         const int j0 = j * panel;
@@ -389,6 +495,7 @@ static cudaError_t launch_factor_wide(Ctx& c) {
         }
       }
     }
+    if (e == cudaSuccess && c.half_rows) next_plane(c.Lmax);   // the last plane's half rows
     // the split buffers are released once the factor's work has completed
     if (Lbuf || Rbuf) {
       cudaStreamSynchronize(c.stream);
@@ -400,19 +507,28 @@ static cudaError_t launch_factor_wide(Ctx& c) {
     if (ev_a) cudaEventDestroy(ev_a);
     if (ev_b) cudaEventDestroy(ev_b);
     if (aux) cudaStreamDestroy(aux);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (W) c.mem.put(W);
     if (e != cudaSuccess) return e;
   } else {
-    for (int k = 0; k < c.Lmax; ++k) {
-      k_plane_schur<C><<<gs, 256, 0, c.stream>>>(c.d_subs, lc, c.node_elems, fac, c.dim, k);
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; e == cudaSuccess && k < c.Lmax; ++k) {
+      next_plane(k);
       for (int j0 = 0; j0 < c.bmax; j0 += panel) {
-        k_gj_panel<C><<<nsub, 256, 0, c.stream>>>(c.d_subs, fac, k, j0, c.d_status);
-        k_gj_rows<C><<<dim3((c.bmax + 127) / 128, nsub), 128, 0, c.stream>>>(c.d_subs, fac, k, j0);
-        k_gj_update<C, T><<<dim3(tiles, tiles, nsub), 256, 0, c.stream>>>(c.d_subs, fac, k, j0);
-        k_gj_cols<C><<<dim3((c.bmax + 127) / 128, nsub), 128, 0, c.stream>>>(c.d_subs, fac, k, j0);
+        k_gj_panel<C><<<nsub, 256, 0, c.stream>>>(subs, fac, k, j0, c.d_status);
+        k_gj_rows<C><<<dim3((c.bmax + 127) / 128, nsub), 128, 0, c.stream>>>(subs, fac, k, j0);
+        k_gj_update<C, T><<<dim3(tiles, tiles, nsub), 256, 0, c.stream>>>(subs, fac, k, j0);
+        k_gj_cols<C><<<dim3((c.bmax + 127) / 128, nsub), 128, 0, c.stream>>>(subs, fac, k, j0);
       }
-      cudaError_t e = cudaGetLastError();
-      if (e != cudaSuccess) return e;
+      e = cudaGetLastError();
     }
+    if (c.half_rows) {
+      if (e == cudaSuccess) next_plane(c.Lmax);
+      if (e == cudaSuccess) e = cudaGetLastError();
+      cudaStreamSynchronize(c.stream);
+      c.mem.put(W);
+    }
+    if (e != cudaSuccess) return e;
   }
   c.kernels += (long long)c.Lmax * (1 + 4 * ((c.bmax + panel - 1) / panel));
   return cudaSuccess;
@@ -426,9 +542,8 @@ bool factor_fits_smem(const Ctx& c) {
 }
 
 cudaError_t launch_factor(Ctx& c) {
-  if (!factor_fits_smem(c))
-    return c.c64() ? launch_factor_wide<float2>(c)
-                                       : launch_factor_wide<double2>(c);
+  if (c.half_rows || !factor_fits_smem(c))
+    return c.c64() ? launch_factor_wide<float2>(c) : launch_factor_wide<double2>(c);
   int nsub = (int)c.subs.size();
   int th = 512;
   if (c.c64()) {

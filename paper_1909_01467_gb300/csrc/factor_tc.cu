@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(tcg::THREADS, tma::Pipe<ES, TERMS>::kCtas) k_g
 
 // The panel inverse of panel columns [j0, j0 + 128) of plane k, every beam, on `stream`.
 cudaError_t launch_gj_panel_inverse(Ctx& c, int k, int j0, cudaStream_t stream) {
-  k_gj_panel_wide<<<(int)c.subs.size(), 512, 0, stream>>>(c.d_subs, reinterpret_cast<float2*>(c.d_fac),
+  k_gj_panel_wide<<<(int)c.subs.size(), 512, 0, stream>>>(c.f_subs, reinterpret_cast<float2*>(c.f_fac),
                                                           k, j0, c.d_status);
   return cudaGetLastError();
 }
@@ -703,7 +703,7 @@ cudaError_t launch_split_panel(Ctx& c, int k, int j0, const SplitJobs& jobs, voi
   return with_form(precision, [&](auto T, auto E) {
     constexpr int TERMS = decltype(T)::value, ES = decltype(E)::value;
     k_split_panel<TERMS, ES><<<dim3(blocks, tma::NCH, (unsigned)c.subs.size()), 256, 0, stream>>>(
-        c.d_subs, reinterpret_cast<const float2*>(c.d_fac), k, j0, jobs,
+        c.f_subs, reinterpret_cast<const float2*>(c.f_fac), k, j0, jobs,
         static_cast<unsigned char*>(L), static_cast<unsigned char*>(R), Lstride, Rstride);
     return cudaGetLastError();
   });
@@ -739,8 +739,8 @@ cudaError_t launch_gj_panel_product_tma(Ctx& c, int k, int j0, int mode, int x0,
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_gemm_panel_tma<TERMS, ES>, c.d_subs,
-                              reinterpret_cast<float2*>(c.d_fac), k, j0, mode,
+    return cudaLaunchKernelEx(&cfg, k_gemm_panel_tma<TERMS, ES>, c.f_subs,
+                              reinterpret_cast<float2*>(c.f_fac), k, j0, mode,
                               mode == 1 ? x0 : 0, x_skip,
                               static_cast<const unsigned char*>(L),
                               static_cast<const unsigned char*>(R), Lstride, Rstride, c.d_status);

@@ -117,7 +117,8 @@ struct SubGeom {
   int gx0, gy0, gz0;     // extended-grid index of the local origin
   int ox0, ox1, oy0, oy1;  // owned range in local coordinates (x, y); z: see oz0, oz1
   int L, b, bp;          // lines (2D: rows y; 3D: planes z), nodes per line, padded b
-  int bs;                // elements per stored block: b + 2 rows of bp (D_k^-1, l_k, l_{k-1})
+  int bs;                // elements per stored block: b + 2 rows of bp (D_k^-1, l_k, l_{k-1}), or
+                         // half_stride(b) in a plan of half rows
   int ax_tab, ay_tab, az_tab;  // offsets of this box's alpha tables (nodes; faces follow)
   long long fac_off;     // element offset of D_0^-1 in the factor array
   long long node_off;    // element offset in the per-node coefficient arrays
@@ -273,6 +274,15 @@ __device__ __host__ inline int tile_index(int b, TileStore s, int es, int r, int
          (i * (i + 1) / 2 + j) * diag_count(G, s.NQ, qd) + d;
 }
 
+// Half rows of a symmetric block (the wide sweep kernel): row r holds the columns r, r + 1, ..,
+// r + b / 2 (mod b), padded to an even count (for even b the pair r, r + b / 2 is in two rows:
+// zero in the later one), so that each unordered pair is there once; the rows are followed by
+// the couplings c_k and c_{k-1}, each padded to an even count, so that every row starts on 16
+// bytes.
+__device__ __host__ inline int half_row(int b) { return (b / 2 + 2) & ~1; }
+__device__ __host__ inline int half_cpl(int b) { return b * half_row(b); }
+__device__ __host__ inline int half_stride(int b) { return half_cpl(b) + 2 * ((b + 1) & ~1); }
+
 // Factor blocks one local solve uses, forward and backward: 2 L, less the steps that the
 // sweep kernel skips.  form: 0 no skip (cluster-split kernels), 1 one CTA per solve (forward
 // from line 0; skips forward steps over zero right-hand sides), 2 twisted factors (forward
@@ -319,6 +329,7 @@ struct Ctx {
   bool cube = false;
   std::vector<AxisBlock> zb;
   int n_trace_arr = N_TRACE_ARR;
+  bool half_rows = false;       // the sweeps run on k_front_wide: blocks stored as half rows
   std::vector<SubGeom> subs;
   std::vector<AlphaSeg> segs;   // PML tables: global, then one per x, y (and z) block
   int alpha_entries = 0;
@@ -340,6 +351,12 @@ struct Ctx {
   void* d_lane = nullptr;       // kLanes accumulation lanes of Next, working precision
   void* d_trace = nullptr;      // n_trace_arr * nsub * 2 * trace_W, working precision
   SubGeom* d_subs = nullptr;
+  // where the wide-plane factor kernels work: the stored blocks themselves, or (half rows) one
+  // whole block per subdomain in a workspace, addressed through geometry copies without a
+  // stride per line (d_wsubs)
+  SubGeom* d_wsubs = nullptr;
+  const SubGeom* f_subs = nullptr;
+  void* f_fac = nullptr;
   Task* d_tasks = nullptr;
   AlphaSeg* d_segs = nullptr;   // the PML tables' descriptors (segs)
   Task* d_raw_task = nullptr;   // single task of lsweep_local_solve
@@ -470,6 +487,7 @@ cudaError_t launch_front_multi(Ctx& c, int li, int K, Ctx* const* rhs, const dou
 // message reported by lsweep_last_error(NULL) for calls that have no handle
 void set_global_error(const std::string& msg);
 bool front_pipeline_fits(const Ctx& c);
+bool uses_wide(const Ctx& c);
 // bytes of global line-vector scratch (d_lines) the plan's sweep kernels need (0: none)
 size_t lines_bytes(const Ctx& c);
 // true when lsweep_factor should store twisted factors: sweep-front kernel 0 (automatic) or 3,
