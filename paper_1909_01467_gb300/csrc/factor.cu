@@ -24,17 +24,34 @@ namespace lsw {
 // m+1 (E_k = A_kk - c_k E_{k+1}^-1 c_k), and last the middle line, whose Schur complement
 // takes both neighbours' updates: T_m = A_mm - c_{m-1} D_{m-1}^-1 c_{m-1} - c_m E_{m+1}^-1 c_m.
 // Stored block k holds the inverse of line k's Schur complement and the couplings c_k, c_{k-1}.
-template <typename C>
-__global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restrict__ lcoef,
+// RPL > 0: the blocked inverse for lines of up to 32 RPL nodes (threads and CTAs per SM:
+// simt_threads); 0: the column by column one (complex128, and lines of more than 158 nodes, whose
+// block leaves no room for the scratch).  Up to 96 nodes two CTAs of 256 threads share an SM, so
+// that one's tiles fill the other's steps; wider blocks are alone on theirs and take more warps,
+// as many as leave warp 0 its rows in registers (a scheduler's 16384 over its warps).
+__host__ __device__ constexpr int simt_threads(int rpl) {
+  return rpl == 0 || rpl == 4 ? 512 : rpl == 6 ? 384 : 256;
+}
+template <typename C, int RPL>
+__global__ void __launch_bounds__(simt_threads(RPL), RPL == 2 || RPL == 3 ? 2 : 1)
+k_factor_simt(const SubGeom* __restrict__ subs, const C* __restrict__ lcoef,
                               long long cstride, C* __restrict__ fac, int dim, TileStore ts,
                               int* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const SubGeom g = subs[blockIdx.x];
   const int b = g.b, bp = g.bp, L = g.L, Lx = g.Lx;
   C* M = reinterpret_cast<C*>(smem_raw);
+  // column by column: the column and the row of a step, the interchanges; blocked: its scratch,
+  // the pivot rows and the step of each
   C* f = M + (size_t)bp * b;
   C* prow = f + b;
-  int* perm = reinterpret_cast<int*>(prow + b);
+  int* perm = reinterpret_cast<int*>(RPL ? f + gj_scratch(b, bp) : prow + b);
+  int* step_of = perm + b;
+  // entry (r, c) of the inverse
+  auto inverse = [&](int r, int c) -> C& {
+    if constexpr (RPL > 0) return M[step_of[c] * bp + perm[r]];
+    else return M[(size_t)c * bp + r];
+  };
   const C* d = lcoef + g.node_off;
   const C* cx = d + cstride;
   const C* cy = d + 2 * cstride;
@@ -59,6 +76,7 @@ __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restr
     }
     const long long bstr = twisted ? block_elems(b, ts) : g.bs;
     const C* Dg = fac + g.fac_off + (cg < 0 ? 0 : cg) * bstr;
+    const C* Di = fac + g.fac_off + (ci < 0 ? 0 : ci) * bstr;
     // Schur complement of line k, built in place over the previous inverse
     for (int idx = tid; idx < b * b; idx += nth) {
       int col = idx / b, row = idx - col * b;
@@ -71,7 +89,9 @@ __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restr
       else if (dim == 3 && row == col + Lx) v = cy[kb + col];
       if (ci >= 0) {
         C lr = cl[(size_t)ci * b + row], lc = cl[(size_t)ci * b + col];
-        v = v - cmul(cmul(lr, M[(size_t)col * bp + row]), lc);
+        // (the blocked inverse of a block stored whole stands permuted in M)
+        const C x = RPL == 0 || twisted ? M[(size_t)col * bp + row] : Di[(size_t)row * bp + col];
+        v = v - cmul(cmul(lr, x), lc);
       }
       if (cg >= 0) {
         C lr = cl[(size_t)cg * b + row], lc = cl[(size_t)cg * b + col];
@@ -80,24 +100,49 @@ __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restr
       M[(size_t)col * bp + row] = v;
     }
     __syncthreads();
-    gauss_jordan_inverse<C>(M, b, bp, f, prow, perm, status);
+    if constexpr (RPL > 0) gj_block_inverse<RPL>(M, b, bp, f, perm, step_of, status);
+    else gauss_jordan_inverse<C>(M, b, bp, f, prow, perm, status);
     C* Dk = fac + g.fac_off + k * bstr;
     if (twisted) {
       // the tiles of the symmetric part, which replaces the inverse in M as well: the next
       // line's Schur complement is then that of the stored block.  n: b padded to whole tiles
-      const int n = tile_rows(b, ts.T) * ts.T;
-      for (int idx = tid; idx < n * (n + 1) / 2; idx += nth) {
+      const int n = tile_rows(b, ts.T) * ts.T, pairs = n * (n + 1) / 2;
+      auto pair = [&](int idx, int& row, int& col) {
         // pair idx of the triangle, two columns of it folded into one of n + 1 entries
         const int j = idx / (n + 1), i = idx - j * (n + 1);
-        const int row = i > j ? i - 1 : n / 2 + j, col = i > j ? j : n / 2 + i;
+        row = i > j ? i - 1 : n / 2 + j;
+        col = i > j ? j : n / 2 + i;
+      };
+      auto store = [&](int idx) {
+        int row, col;
+        pair(idx, row, col);
         C v = czero<C>();
         if (row < b) {
-          const C u = M[(size_t)col * bp + row], t = M[(size_t)row * bp + col];
+          const C u = inverse(row, col), t = inverse(col, row);
           v = mk((u.x + t.x) / 2, (u.y + t.y) / 2);
-          M[(size_t)col * bp + row] = v;
-          M[(size_t)row * bp + col] = v;
         }
         Dk[tile_index(b, ts, (int)sizeof(C), row, col)] = v;
+        return v;
+      };
+      auto put = [&](int idx, C v) {
+        int row, col;
+        pair(idx, row, col);
+        if (row < b) M[(size_t)col * bp + row] = M[(size_t)row * bp + col] = v;
+      };
+      if constexpr (RPL > 0) {
+        // the pairs leave their permuted places in registers before any is written in its own
+        constexpr int NM = RPL == 6 ? 168 : 32 * RPL + 5;
+        constexpr int NP = (NM * (NM + 1) / 2 + simt_threads(RPL) - 1) / simt_threads(RPL);
+        C v[NP];
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+          if (tid + i * nth < pairs) v[i] = store(tid + i * nth);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+          if (tid + i * nth < pairs) put(tid + i * nth, v[i]);
+      } else {
+        for (int idx = tid; idx < pairs; idx += nth) put(idx, store(idx));
       }
       const int bs = (b + 1) & ~1;
       for (int q = 0; q < ts.NQ; ++q) {
@@ -115,7 +160,7 @@ __global__ void k_factor_simt(const SubGeom* __restrict__ subs, const C* __restr
       int row = idx / bp, col = idx - row * bp;
       C v = czero<C>();
       if (col < b) {
-        if (row < b) v = M[(size_t)col * bp + row];
+        if (row < b) v = inverse(row, col);
         else if (row == b) v = cl[(size_t)k * b + col];                       // c_k
         else if (k > 0) v = cl[(size_t)(k - 1) * b + col];                   // c_{k-1}
       }
@@ -535,37 +580,33 @@ static cudaError_t launch_factor_wide(Ctx& c) {
 }
 
 // planes whose Gauss-Jordan block fits in shared memory use k_factor_simt
-bool factor_fits_smem(const Ctx& c) {
+static size_t simt_smem(const Ctx& c, int rpl) {
   const size_t es = c.c64() ? sizeof(float2) : sizeof(double2);
-  const size_t smem = (size_t)c.bpmax * c.bmax * es + 2 * c.bmax * es + c.bmax * sizeof(int) + 16;
-  return smem <= 227 * 1024;
+  const size_t work = rpl ? gj_scratch(c.bmax, c.bpmax) * es + 2 * c.bmax * sizeof(int)
+                          : 2 * c.bmax * es + c.bmax * sizeof(int);
+  return (size_t)c.bpmax * c.bmax * es + work + 16;
 }
+bool factor_fits_smem(const Ctx& c) { return simt_smem(c, 0) <= 227 * 1024; }
 
 cudaError_t launch_factor(Ctx& c) {
   if (c.half_rows || !factor_fits_smem(c))
     return c.c64() ? launch_factor_wide<float2>(c) : launch_factor_wide<double2>(c);
-  int nsub = (int)c.subs.size();
-  int th = 512;
-  if (c.c64()) {
-    size_t smem = (size_t)c.bpmax * c.bmax * sizeof(float2) + 2 * c.bmax * sizeof(float2) +
-                  c.bmax * sizeof(int) + 16;
-    cudaError_t e = cudaFuncSetAttribute(k_factor_simt<float2>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const TileStore ts = c.fac_twisted ? tile_store(c) : TileStore{0, 1};
+  auto launch = [&](auto kern, auto zero, int rpl) {
+    using C = decltype(zero);
+    const size_t smem = simt_smem(c, rpl);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_factor_simt<float2><<<nsub, th, smem, c.stream>>>(c.d_subs, (const float2*)c.d_lcoef,
-                                                        c.node_elems, (float2*)c.d_fac, c.dim,
-                                                        c.fac_twisted ? tile_store(c) : TileStore{0, 1}, c.d_status);
-  } else {
-    size_t smem = (size_t)c.bpmax * c.bmax * sizeof(double2) + 2 * c.bmax * sizeof(double2) +
-                  c.bmax * sizeof(int) + 16;
-    cudaError_t e = cudaFuncSetAttribute(k_factor_simt<double2>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_factor_simt<double2><<<nsub, th, smem, c.stream>>>(c.d_subs, (const double2*)c.d_lcoef,
-                                                         c.node_elems, (double2*)c.d_fac, c.dim,
-                                                         c.fac_twisted ? tile_store(c) : TileStore{0, 1}, c.d_status);
-  }
-  return cudaGetLastError();
+    kern<<<(unsigned)c.subs.size(), simt_threads(rpl), smem, c.stream>>>(
+        c.d_subs, (const C*)c.d_lcoef, c.node_elems, (C*)c.d_fac, c.dim, ts, c.d_status);
+    return cudaGetLastError();
+  };
+  if (!c.c64()) return launch(k_factor_simt<double2, 0>, double2(), 0);
+  if (simt_smem(c, 6) > 227 * 1024) return launch(k_factor_simt<float2, 0>, float2(), 0);
+  if (c.bmax <= 64) return launch(k_factor_simt<float2, 2>, float2(), 2);
+  if (c.bmax <= 96) return launch(k_factor_simt<float2, 3>, float2(), 3);
+  if (c.bmax <= 128) return launch(k_factor_simt<float2, 4>, float2(), 4);
+  return launch(k_factor_simt<float2, 6>, float2(), 6);
 }
 
 }  // namespace lsw

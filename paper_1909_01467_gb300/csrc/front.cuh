@@ -28,7 +28,7 @@ struct FrontArgs {
   const double2* rin;    // stage 1 input (extended grid)
   const double2* g_raw;  // RAW: local right-hand side
   double2* x_raw;        // RAW: local solution
-  long long spin;        // limit of a dependency wait (cycles) in kernels solo / pair / quad
+  long long spin;        // limit of a dependency wait (cycles) in the sweep kernels
   int skip;              // fused applications: 1 = this problem is not applied (CTAs exit)
 };
 
