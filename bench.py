@@ -389,7 +389,7 @@ def run_ours(args):
                          "(4 FGMRES(30) processes sharing block applications) to 1e-8",
                  "roofline": {"bound": "hbm", "achieved": ach_m, "peak": peak_m, "unit": "GB/s",
                               "frac": ach_m / peak_m if ach_m else None, "traffic": None,
-                              "kernel": "k_front_pair_multi (block of the active right-hand "
+                              "kernel": "k_twist_multi (block of the active right-hand "
                                         "sides per factor block; bytes: the factor stream of "
                                         "one application per block application)",
                               "block_applications": int(pm.front_launches // max(1, h_levels(L, h)))},
@@ -420,14 +420,15 @@ def run_ours(args):
         c128_roof = None
         peak_hbm, peak_src = measured_peak_hbm()
         if pc.front_ms > 0:
-            # each complex128 factor entry streamed (16 B) is one complex multiply-add of the
-            # block-vector product: 4 FP64 FMAs, 8 flops; GB300's FP64 rate bounds this form
-            flops = pc.front_bytes / 16 * 8
+            # each complex128 factor entry streamed (16 B) stands for a pair of the symmetric
+            # block: two complex multiply-adds, 8 FP64 FMAs, 16 flops; GB300's FP64 rate bounds
+            # this form
+            flops = pc.front_bytes / 16 * 16
             ach = flops / (pc.front_ms / 1e3) / 1e12
             gbs = pc.front_bytes / (pc.front_ms / 1e3) / 1e9
             c128_roof = {"bound": "alu", "achieved": ach, "peak": FP64_TFLOPS, "unit": "TFLOP/s",
                          "frac": ach / FP64_TFLOPS, "traffic": None,
-                         "kernel": "k_front_quad<double2> (four CTAs per local solve on the "
+                         "kernel": "k_twist_rows (four CTAs per local solve on the "
                                    "twisted factor, line vectors in global memory): FP64 "
                                    "block-vector products",
                          "peak_source": "nominal GB300 FP64 rate (no measured FP64 peak)",
@@ -491,7 +492,7 @@ def run_ours(args):
                    "n": n, "npml": w.npml, "cdd": list(w.cdd),
                    "omega": w.omega, "sources": len(srcs), "precision": "mixed",
                    "step": "coefficients + factor + 4 FGMRES(30) solves to 1e-8",
-                   "l2": "inputs larger than L2 (factors 1.6 GB streamed per apply)",
+                   "l2": "inputs larger than L2 (factors 0.9 GB streamed per apply)",
                    "parallelism": f"replicas x{world}", "front_kernel": args.front_kernel,
                    "pdl": not args.no_pdl},
         "iterations": iters[: len(srcs)],
@@ -508,10 +509,10 @@ def run_ours(args):
                      "traffic": front_traffic(n, args.front_kernel),
                      "kernel": {1: "k_front (cluster split)",
                                 2: "k_front_solo (one CTA per local solve)",
-                                3: "k_front_pair (two CTAs per local solve, twisted factor)"}.get(
+                                3: "k_twist (two CTAs per local solve, twisted factor)"}.get(
                                     args.front_kernel,
-                                    "k_front_pair / k_front_quad (two CTAs per local solve on "
-                                    "the twisted factor, four on levels of few solves)") +
+                                    "k_twist (two CTAs per local solve on the twisted "
+                                    "factor, stored as triangles)") +
                                ": transfer source + block substitution",
                      "peak_source": peak_src,
                      "front_launches": prof.front_launches,
@@ -625,7 +626,9 @@ def batch_record(args) -> dict:
             L.lsweep_solve_batch(handles, fs, us)
         torch.cuda.synchronize()
         unknowns = sum(n * n for n, _, _, _ in probs)
-        fac_bytes = [L.lsweep_factor_bytes(h)[1] for h in handles]
+        # (whole blocks; the twisted kernels, 0 and 3, stream the triangles: half of them)
+        share = 0.5 if tuned["kernel"] in (0, 3) else 1.0
+        fac_bytes = [share * L.lsweep_factor_bytes(h)[1] for h in handles]
         clocks = Clocks()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         torch.cuda.synchronize()
@@ -792,7 +795,7 @@ def layered3d_record(args, cube=False) -> dict:
                    "planes": h.Ne, "factor_bytes": stored,
                    "precision": getattr(args, "precision3d", PRECISION3D),
                    "prefetch_chunks": args.prefetch_steps,
-                   "l2": "inputs larger than L2 (factors %.1f GB streamed per apply)" % (per_apply / 1e9)},
+                   "l2": "inputs larger than L2 (factors %.1f GB streamed per apply)" % (per_apply / 2e9)},
         "iterations": its[: args.steps], "factor_ms": prof.factor_ms,
         "factor": {"flops": flops, "ms": prof.factor_ms,
                    "tflops": flops / (prof.factor_ms / 1e3) / 1e12 if prof.factor_ms else None},
@@ -800,7 +803,7 @@ def layered3d_record(args, cube=False) -> dict:
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak if achieved else None, "traffic": None,
                      "peak_source": peak_src,
-                     "kernel": "k_front_wide (cluster per solve, chunked rows) timed per "
+                     "kernel": "k_front_wide (cluster per solve, chunks of half rows) timed per "
                                "application (graph replay)",
                      "front_launches": prof.front_launches},
         "clocks": clk, "cpu_baseline": None, "e2e": None,
