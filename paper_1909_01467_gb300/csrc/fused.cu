@@ -4,7 +4,8 @@
 // application is captured once as a CUDA graph and replayed.  The problems' inputs and
 // outputs change from application to application (the FGMRES basis vectors), so the graph
 // reads them from a device table that is refreshed before each replay, with a flag that
-// leaves out the problems that are not applied (converged solves): their CTAs exit at once.
+// leaves out the problems that are not applied (converged solves): their CTAs only wait for the
+// previous level, which keeps the chain of levels whole.
 // Requires problems with the same sweep-front geometry (line width, padded width, lines)
 // and the same kernel form (twisted factors, or one CTA per solve),
 // complex64.  lsweep_solve_batch_fused runs the problems' FGMRES processes in lockstep on

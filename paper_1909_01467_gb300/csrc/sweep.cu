@@ -219,7 +219,10 @@ __global__ void __launch_bounds__(768, 1) k_front_solo(FrontArgs a_, int Lmax, i
   griddep_launch_dependents();                          // the next level may start its setup
   const Task task = a_.tasks[a_.task_off + blockIdx.x];
   const FrontArgs& a = kFused ? table[task.kind >> 8] : a_;
-  if (kFused && a.skip) return;
+  if (kFused && a.skip) {                               // (waits: as in k_twist)
+    griddep_wait();
+    return;
+  }
   const int sub = task.sub, kind = kFused ? (task.kind & 0xff) : task.kind;
   const SubGeom g = a.subs[sub];
   const int b = g.b, bp = g.bp, L = g.L;

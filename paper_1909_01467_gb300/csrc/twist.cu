@@ -451,7 +451,7 @@ __device__ void dense_source(const FrontArgs& a, const SubGeom& g, int kind, C* 
 // (1 - h, q).
 // kFused: one launch over the solves of several problems (fused applications): the task's
 // kind carries its problem in bits 8.., whose arguments come from `table`; a problem marked
-// skip is not applied (its CTAs exit at once).
+// skip is not applied (its CTAs wait for the previous level and exit).
 template <int T, int GM, int NQ, bool kFused>
 __global__ void __launch_bounds__(twist_threads(T, GM, NQ), 1)
 k_twist(FrontArgs a_, Twist tg, const FrontArgs* __restrict__ table, int* status) {
@@ -462,7 +462,12 @@ k_twist(FrontArgs a_, Twist tg, const FrontArgs* __restrict__ table, int* status
   griddep_launch_dependents();                          // the next level may start its setup
   const Task task = a_.tasks[a_.task_off + blockIdx.x / (2 * NQ)];
   const FrontArgs& a = kFused ? table[task.kind >> 8] : a_;
-  if (kFused && a.skip) return;
+  if (kFused && a.skip) {
+    // (a level is complete only with the levels before it: a launch of nothing but such CTAs must
+    // not finish while an earlier one still runs, as the next launch waits for this one alone)
+    griddep_wait();
+    return;
+  }
   const int sub = task.sub, kind = kFused ? (task.kind & 0xff) : task.kind;
   const SubGeom g = a.subs[sub];
   const int b = g.b, L = g.L, G = tile_rows(b, T);
