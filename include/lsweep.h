@@ -389,7 +389,10 @@ int lsweep_ext_size(lsweep_handle h, int64_t* n_ext);
  * subdomain, 2 L b^2 element sizes less the block steps that the kernel skips (forward over
  * lines where the right-hand side is zero: one-CTA and twisted kernels; backward past the last
  * line that is read: twisted kernels).  Twisted factors store and stream the triangle of each
- * block, (b + 1) / (2 b) of this (lsweep_profile.front_bytes).  Host outputs. */
+ * block, (b + 1) / (2 b) of this, and the kernel of planes too wide for a row slab half rows, as
+ * many bytes (lsweep_profile.front_bytes).  A plan that the twisted kernels take holds
+ * room for whole blocks as well, which lsweep_autotune may change to: its allocation is the larger
+ * of the two forms, not the stored bytes.  Host outputs. */
 int lsweep_factor_bytes(lsweep_handle h, int64_t* stored, int64_t* per_apply);
 
 /* Result of lsweep_autotune (host struct). */
@@ -430,7 +433,8 @@ typedef struct lsweep_profile {
                             /* its trace reset and lane sum included)                     */
   double front_bytes;       /* factor bytes those launches must stream: per subdomain      */
                             /* visited, forward and backward, whole blocks of b^2 entries  */
-                            /* or (twisted factors) their triangles, skipped steps left out */
+                            /* or (twisted factors, half rows) half of each, skipped steps  */
+                            /* left out                                                    */
   double factor_ms;         /* duration of the last lsweep_factor (CUDA events)           */
 } lsweep_profile;
 

@@ -430,9 +430,7 @@ int build_plan(Ctx* c) {
       g.ax_tab = xtab[j];
       g.ay_tab = ytab[i];
       g.az_tab = ztab[k];
-      g.fac_off = fac;
       g.node_off = node;
-      fac += (long long)g.L * g.bs;
       node += (long long)g.L * g.b;
       c->Lmax = std::max(c->Lmax, g.L);
       c->bmax = std::max(c->bmax, g.b);
@@ -442,15 +440,13 @@ int build_plan(Ctx* c) {
       c->subs.push_back(g);
     }
   }
-  // plans whose sweeps stream half rows store those
+  // plans whose sweeps stream half rows store those, the others whole blocks or triangles
   c->half_rows = lsw::uses_wide(*c);
-  if (c->half_rows) {
-    fac = 0;
-    for (auto& g : c->subs) {
-      g.bs = lsw::half_stride(g.b);
-      g.fac_off = fac;
-      fac += (long long)g.L * g.bs;
-    }
+  const lsw::TileStore ts = lsw::twist_fits(*c) ? lsw::tile_store(*c) : lsw::TileStore{0, 1};
+  for (auto& g : c->subs) {
+    if (c->half_rows) g.bs = lsw::half_stride(g.b);
+    g.fac_off = fac;
+    fac += (long long)g.L * (c->half_rows ? g.bs : lsw::block_room(g.b, g.bs, ts));
   }
   c->fac_elems = fac;
   c->node_elems = node;
@@ -1291,12 +1287,11 @@ int lsweep_ext_size(lsweep_handle h, int64_t* n_ext) {
 int lsweep_factor_bytes(lsweep_handle h, int64_t* stored, int64_t* per_apply) {
   Ctx* c = (Ctx*)h;
   if (!c || !stored || !per_apply) return LSWEEP_EINVAL;
-  int64_t elems = c->fac_elems;
-  if (c->twisted()) {
-    elems = 0;
-    const lsw::TileStore st = lsw::tile_store(*c);
-    for (const auto& g : c->subs) elems += (int64_t)g.L * lsw::block_elems(g.b, st);
-  }
+  int64_t elems = 0;
+  const bool tri = c->twisted();
+  const lsw::TileStore st = tri ? lsw::tile_store(*c) : lsw::TileStore{0, 1};
+  for (const auto& g : c->subs)
+    elems += (int64_t)g.L * (tri ? lsw::block_elems(g.b, st) : g.bs);
   *stored = elems * (int64_t)c->welem();
   *per_apply = c->per_apply_elems_f[lsw::front_form(*c)] * (int64_t)c->welem();
   return LSWEEP_OK;

@@ -244,6 +244,17 @@ __device__ __host__ inline int tile_number(int I, int J, int NQ) {
   return (I + J) & 1 ? I * I / 4 + (J - ((I + 1) & 1)) / 2
                      : (I - 1) * (I - 1) / 4 + (J - (I & 1)) / 2;
 }
+// Worker (I, J) of CTA q: its tile number among the CTA's and its indices; none for threads
+// past the last tile.
+template <int NQ>
+__device__ __host__ inline bool worker_tile(int o, int G, int q, int& I, int& J) {
+  I = J = 0;
+  if (o >= tile_count(G, NQ, q)) return false;
+  for (I = 1; I + 1 < G && tile_number(I + 1, NQ == 1 ? 0 : (I + 1 + q) & 1, NQ) <= o; ++I) {}
+  J = o - tile_number(I, NQ == 1 ? 0 : (I + q) & 1, NQ);
+  if (NQ == 2) J = 2 * J + ((I + q) & 1);
+  return true;
+}
 __device__ __host__ inline int part_cpl(int b, TileStore s, int q) {   // offset of the couplings
   const int G = tile_rows(b, s.T);
   return tile_count(G, s.NQ, q) * s.T * s.T +
@@ -254,6 +265,13 @@ __device__ __host__ inline int part_elems(int b, TileStore s, int q) {
 }
 __device__ __host__ inline int block_elems(int b, TileStore s) {
   return part_elems(b, s, 0) + (s.NQ > 1 ? part_elems(b, s, 1) : 0);
+}
+// Entries that the plan sets aside per stored block of `whole` entries ((b + 2) rows of bp): the
+// blocks of a plan that the twisted kernels take may be stored in either form (lsweep_autotune
+// moves between them), and for lines of 2 and 5 nodes the padded tiles are the larger one.
+__device__ __host__ inline long long block_room(int b, int whole, TileStore s) {
+  const int tri = s.T ? block_elems(b, s) : 0;
+  return tri > whole ? tri : whole;
 }
 // entry (r, c) of a block whose entries are es bytes (8 or 16)
 __device__ __host__ inline int tile_index(int b, TileStore s, int es, int r, int c) {

@@ -80,18 +80,6 @@ __device__ inline void load_run(const float2* p, float2 (&v)[T]) {
 __device__ inline void store_pair(float2* p, float2 a, float2 b) {
   *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
 }
-// Worker (I, J) of CTA q: its tile number among the CTA's and its indices; none for threads
-// past the last tile.
-template <int NQ>
-__device__ inline bool worker_tile(int o, int G, int q, int& I, int& J) {
-  I = J = 0;
-  if (o >= tile_count(G, NQ, q)) return false;
-  for (I = 1; I + 1 < G && tile_number(I + 1, NQ == 1 ? 0 : (I + 1 + q) & 1, NQ) <= o; ++I) {}
-  J = o - tile_number(I, NQ == 1 ? 0 : (I + q) & 1, NQ);
-  if (NQ == 2) J = 2 * J + ((I + q) & 1);
-  return true;
-}
-
 // Rows i, i + 1 of this thread's tile from a ring slot.
 template <int T>
 __device__ __forceinline__ void load_rows(float2 (&D)[T * T], const unsigned char* tile,
