@@ -450,16 +450,25 @@ static cudaError_t launch_factor_wide(Ctx& c) {
   const C* lc = reinterpret_cast<const C*>(c.d_lcoef);
   const long long bs_max = (long long)(c.bmax + 2) * c.bpmax;
   const dim3 gs((unsigned)std::min<long long>(1024, (bs_max + 255) / 256), (unsigned)nsub);
+  // complex64: 128-column panels with the products on the tensor cores (three TF32 terms
+  // per operand: FP32-level; one for LSWEEP_C64_TF32; three BF16 terms for
+  // LSWEEP_C64_BF16X3); complex128: 32-column panels on the CUDA cores in FP64
+  constexpr bool tc = std::is_same<C, float2>::value;
+  if (tc) {
+    cudaError_t e = prepare_gj_panel_tc();
+    if (e != cudaSuccess) return e;
+  }
   // whole blocks are inverted where they are stored; half rows are made from one whole block
   // per subdomain in a workspace, which every plane passes through
   void* W = nullptr;
-  c.f_subs = c.half_rows ? c.d_wsubs : c.d_subs;
-  c.f_fac = c.d_fac;
+  void* fac_at = c.d_fac;
   if (c.half_rows) {
     W = c.mem.get((size_t)nsub * c.bmax * c.bpmax * sizeof(C));
     if (!W) return cudaErrorMemoryAllocation;
-    c.f_fac = W;
+    fac_at = W;
   }
+  c.f_subs = c.half_rows ? c.d_wsubs : c.d_subs;
+  c.f_fac = fac_at;
   C* fac = reinterpret_cast<C*>(c.f_fac);
   const SubGeom* subs = c.f_subs;
   const unsigned t32 = (unsigned)((c.bmax + 31) / 32);
@@ -471,16 +480,8 @@ static cudaError_t launch_factor_wide(Ctx& c) {
     else
       k_plane_schur<C><<<gs, 256, 0, c.stream>>>(subs, lc, c.node_elems, fac, c.dim, k);
   };
-  // complex64: 128-column panels with the products on the tensor cores (three TF32 terms
-  // per operand: FP32-level; one for LSWEEP_C64_TF32; three BF16 terms for
-  // LSWEEP_C64_BF16X3); complex128: 32-column panels on the CUDA cores in FP64
-  constexpr bool tc = std::is_same<C, float2>::value;
-
   const int panel = tc ? gj_panel_width_tc() : kPanel;
-  if (tc) {
-    cudaError_t e = prepare_gj_panel_tc();
-    if (e != cudaSuccess) return e;
-  }
+  cudaError_t e = cudaSuccess;
   constexpr int T = 32;
   const int tiles = (c.bmax + T - 1) / T;
   const int npan = (c.bmax + panel - 1) / panel;
@@ -492,7 +493,7 @@ static cudaError_t launch_factor_wide(Ctx& c) {
     // columns, so column tile j + 1 is panel j + 1.
     cudaStream_t aux = nullptr;
     cudaEvent_t ev_a = nullptr, ev_b = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&aux, cudaStreamNonBlocking);
+    e = cudaStreamCreateWithFlags(&aux, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_a, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_b, cudaEventDisableTiming);
     const int prec = c.p.precision;
@@ -541,22 +542,17 @@ static cudaError_t launch_factor_wide(Ctx& c) {
       }
     }
     if (e == cudaSuccess && c.half_rows) next_plane(c.Lmax);   // the last plane's half rows
-    // the split buffers are released once the factor's work has completed
-    if (Lbuf || Rbuf) {
-      cudaStreamSynchronize(c.stream);
-      if (Lbuf) c.mem.put(Lbuf);
-      if (Rbuf) c.mem.put(Rbuf);
-    }
-    // the last aux work was joined into c.stream; the stream and events are released once
-    // their work completes
+    if (e == cudaSuccess) e = cudaGetLastError();
+    // the buffers are released once the factor's work has completed, on both streams: after an
+    // error the last work of aux may not have been joined into c.stream
+    cudaStreamSynchronize(c.stream);
+    if (aux) cudaStreamSynchronize(aux);
+    c.mem.put(Lbuf);
+    c.mem.put(Rbuf);
     if (ev_a) cudaEventDestroy(ev_a);
     if (ev_b) cudaEventDestroy(ev_b);
     if (aux) cudaStreamDestroy(aux);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (W) c.mem.put(W);
-    if (e != cudaSuccess) return e;
   } else {
-    cudaError_t e = cudaSuccess;
     for (int k = 0; e == cudaSuccess && k < c.Lmax; ++k) {
       next_plane(k);
       for (int j0 = 0; j0 < c.bmax; j0 += panel) {
@@ -571,10 +567,12 @@ static cudaError_t launch_factor_wide(Ctx& c) {
       if (e == cudaSuccess) next_plane(c.Lmax);
       if (e == cudaSuccess) e = cudaGetLastError();
       cudaStreamSynchronize(c.stream);
-      c.mem.put(W);
     }
-    if (e != cudaSuccess) return e;
   }
+  c.mem.put(W);
+  c.f_subs = nullptr;
+  c.f_fac = nullptr;
+  if (e != cudaSuccess) return e;
   c.kernels += (long long)c.Lmax * (1 + 4 * ((c.bmax + panel - 1) / panel));
   return cudaSuccess;
 }
