@@ -45,6 +45,7 @@ struct Twist {
   TileStore ts;
   int Lh, bs;            // lines per half at most; bmax rounded up to even
   int nslot, PD;         // ring slots; steps between a copy and the L2 prefetch it issues
+  int W;                 // k_twist_rows: consumer warps
   unsigned slot_bytes;
 };
 
@@ -746,19 +747,20 @@ k_twist(FrontArgs a_, Twist tg, const FrontArgs* __restrict__ table, int* status
 // The same solve with FP64 products, which two lanes a clock per SM bound (a warp's multiply-
 // add keeps its scheduler's FP64 unit busy for 64 clocks however many lanes are active).  So a
 // block's rows are split over two CTAs per half, and the row and column split inside a CTA is
-// chosen to fill 12 warps, three per scheduler, with as few idle lanes as possible: thread t
-// has row t mod nr and column chunk t / nr, CH = 384 / nr chunks.  Every CTA copies whole
+// chosen to fill its W warps with as few idle lanes as possible: thread t has row t mod nr and
+// column chunk t / nr, CH = 32 W / nr chunks (W = 12: three warps per scheduler; shorter lines take
+// 6 warps and two CTAs per SM or 3 and four, see rows_warps).  Every CTA copies whole
 // stored blocks; a thread's entries have fixed offsets in the slot, and those of step s + 1
 // are read while step s is finished.  CTA (h, q) owns rows [q RB, q RB + nr) of its half's
 // line vectors; the owners send their entries of the next vector to the mate (st.async, two
 // barriers by step parity, re-armed one step ahead), and at the last step before the middle
 // line their part of its right-hand side to both CTAs of the other half.
-constexpr int kRowsWarps = 12, kRowsMaxCH = 32;
-template <int NC>
-__global__ void __launch_bounds__(kRowsWarps * 32 + 32, 1)
+constexpr int kRowsMaxCH = 32;
+template <int W, int NC>
+__global__ void __launch_bounds__(W * 32 + 32, 12 / W)
 k_twist_rows(FrontArgs a, Twist tg, int* status) {
   using C = double2;
-  constexpr int ncons = kRowsWarps * 32;
+  constexpr int ncons = W * 32;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   griddep_launch_dependents();                          // the next level may start its setup
   const Task task = a.tasks[a.task_off + blockIdx.x / 4];
@@ -780,7 +782,7 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   const int ka = h ? m : 0, kb = h ? L : m + 1;        // lines of this half (m in both)
   const int CH = min(kRowsMaxCH, ncons / RB), nc = (b + CH - 1) / CH;
   // shared memory: ring[nslot][slot_bytes] | full[8] | empty[8] | vbar[2] | xbar[2] | flags[4]
-  // (32-bit) | vb[2][bs] | part[384] | xb[bs] | H[2][bs] | V[2][Lh] | yl[Lh][RB]
+  // (32-bit) | vb[2][bs] | part[32 W] | xb[bs] | H[2][bs] | V[2][Lh] | yl[Lh][RB]
   unsigned char* ring = smem_raw;
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)tg.nslot * tg.slot_bytes);
   uint64_t* empty = full + kSoloMaxSlots;
@@ -819,7 +821,7 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   if (tid == 0) {
     for (int i = 0; i < tg.nslot; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], kRowsWarps);
+      mbar_init(&empty[i], W);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&vbar[i], 1);
@@ -836,7 +838,7 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   }
   __syncthreads();
   cluster_sync_all();                                  // every CTA's barriers are armed
-  if (w == kRowsWarps && lane == 0) {
+  if (w == W && lane == 0) {
     for (int t = 0; t < min(tg.PD, nit); ++t) bulk_prefetch_l2(src(t), blk_bytes);
     for (int t = 0; t < min(tg.nslot, nit); ++t) issue(t, t);
   }
@@ -858,7 +860,7 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   __syncthreads();
 
   int varmed = nit > 2 ? 2 : nit - 1, vok = 0;          // (tid 0) last step armed / received
-  if (w == kRowsWarps) {
+  if (w == W) {
     // ---- producer (as k_twist) ---------------------------------------------------------
     if (lane == 0) {
       int issued = min(tg.nslot, nit);
@@ -1341,6 +1343,19 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
 // 1024^2 workload took 3.3 ms, with 4 x 4 2.9 ms).  Wider lines share tiles of 6 x 6 between
 // two CTAs per half, as whole blocks no longer fit beside the line vectors.  Complex128:
 // k_twist_rows, four CTAs per solve.
+// columns per thread of k_twist_rows with W warps (0: too few threads for the rows)
+static int rows_columns(int b, int W) {
+  const int CH = std::min(kRowsMaxCH, W * 32 / ((b + 1) / 2));
+  return CH < 2 ? 0 : (b + CH - 1) / CH;
+}
+// Warps of k_twist_rows, CTAs per SM 12 / W: 3 on lines of up to 36 nodes, 6 up to 54 (what eight
+// columns per thread cover), 12 above.  Short lines are bound by the solves that run at once where
+// levels are full, and where they are not by the barriers and by the sum over the column chunks,
+// which fewer threads shorten.  ms per application with 12 warps -> with these (the four-CTA kernel
+// on whole blocks): 16 x 16 subdomains of 20-node lines 8.8 -> 2.7 (4.8), 36 nodes 13.5 -> 4.9 (9.9),
+// 52 nodes 17.8 -> 9.0 (17.9); 4 x 4 of 20 nodes 0.96 -> 0.40 (0.53), 36 nodes 1.50 -> 0.64 (1.12),
+// 52 nodes 1.96 -> 1.16 (1.95).  36 nodes with 6 warps: 6.1 and 0.86.
+static bool rows_warps(int b, int W) { return W == 12 || b <= (W == 6 ? 54 : 36); }
 // tile rows at most: lines of up to 64 nodes, up to 96, wider ones on two CTAs per half
 constexpr int kGMs = 16, kGM1 = 24, kGM2 = 26;
 static bool twist_geometry(const Ctx& c, Twist& t, int& GM, int& threads, size_t& smem) {
@@ -1367,27 +1382,31 @@ static bool twist_geometry(const Ctx& c, Twist& t, int& GM, int& threads, size_t
     fixed += ((size_t)2 * t.ts.T * GM + GM * SP + 8 + (t.ts.NQ == 2 ? 3 : 1) * t.bs +
               (size_t)t.Lh * b + 1) * es;
   } else {
-    const int RB = (b + 1) / 2;
     GM = 0;
-    threads = (kRowsWarps + 1) * 32;
-    const int CH = std::min(kRowsMaxCH, kRowsWarps * 32 / RB);
-    if (b < 2 || CH < 2 || (b + CH - 1) / CH > 16) return false;
-    fixed += ((size_t)5 * t.bs + kRowsWarps * 32 + 2 * t.Lh + (size_t)t.Lh * RB) * es;
+    if (b < 2) return false;
+    fixed += ((size_t)5 * t.bs + 2 * t.Lh + (size_t)t.Lh * ((b + 1) / 2)) * es;
+    for (int W : {3, 6, 12}) {
+      const int nc = rows_columns(b, W), per_sm = 12 / W;
+      if (!rows_warps(b, W) || nc < 1 || nc > (W == 12 ? 16 : 8)) continue;
+      const size_t limit = 228 * 1024 / per_sm - 1024, all = fixed + W * 32 * es;
+      if (all + 2 * (size_t)t.slot_bytes > limit) continue;
+      t.W = W;
+      t.nslot = (int)std::min<size_t>(kSoloMaxSlots, (limit - all) / t.slot_bytes);
+      smem = all + (size_t)t.nslot * t.slot_bytes;
+      threads = (W + 1) * 32;
+      return true;
+    }
+    return false;
   }
   const size_t limit = 227 * 1024;
   if (fixed + 2 * (size_t)t.slot_bytes > limit) return false;
+  t.W = 0;
   t.nslot = (int)std::min<size_t>(kSoloMaxSlots, (limit - fixed) / t.slot_bytes);
   smem = fixed + (size_t)t.nslot * t.slot_bytes;
   return true;
 }
 // CTAs of a solve
 static int twist_ctas(const Ctx& c, const Twist& t) { return c.c64() ? 2 * t.ts.NQ : 4; }
-// columns per thread of k_twist_rows (its template parameter)
-static int rows_columns(const Ctx& c) {
-  const int RB = (c.bmax + 1) / 2, CH = std::min(kRowsMaxCH, kRowsWarps * 32 / RB);
-  const int nc = (c.bmax + CH - 1) / CH;
-  return nc <= 8 ? 8 : nc <= 12 ? 12 : 16;
-}
 
 bool twist_fits(const Ctx& c) {
   Twist t;
@@ -1410,12 +1429,14 @@ static TwistKernel twist_kernel(const Ctx& c, const Twist& t, bool fused) {
   return c.bmax <= 64 ? k_twist<4, kGMs, 1, false> : k_twist<4, kGM1, 1, false>;
 }
 using RowsKernel = void (*)(FrontArgs, Twist, int*);
-static RowsKernel rows_kernel(const Ctx& c) {
-  const int nc = rows_columns(c);
-  return nc == 8 ? k_twist_rows<8> : nc == 12 ? k_twist_rows<12> : k_twist_rows<16>;
+static RowsKernel rows_kernel(const Ctx& c, const Twist& t) {
+  if (t.W == 3) return k_twist_rows<3, 8>;
+  if (t.W == 6) return k_twist_rows<6, 8>;
+  const int nc = rows_columns(c.bmax, 12);
+  return nc <= 8 ? k_twist_rows<12, 8> : nc <= 12 ? k_twist_rows<12, 12> : k_twist_rows<12, 16>;
 }
 static const void* twist_function(const Ctx& c, const Twist& t, bool fused) {
-  return c.c64() ? (const void*)twist_kernel(c, t, fused) : (const void*)rows_kernel(c);
+  return c.c64() ? (const void*)twist_kernel(c, t, fused) : (const void*)rows_kernel(c, t);
 }
 
 static void twist_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int ctas, int count,
@@ -1448,7 +1469,7 @@ cudaError_t launch_twist(Ctx& c, const FrontArgs& a, int count, const FrontArgs*
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   twist_config(cfg, at, twist_ctas(c, t), count, th, smem, stream, c.p.pdl != 0);
-  if (!c.c64()) return cudaLaunchKernelEx(&cfg, rows_kernel(c), a, t, c.d_status);
+  if (!c.c64()) return cudaLaunchKernelEx(&cfg, rows_kernel(c, t), a, t, c.d_status);
   return cudaLaunchKernelEx(&cfg, twist_kernel(c, t, table != nullptr), a, t, table, c.d_status);
 }
 
@@ -1466,7 +1487,7 @@ int twist_concurrency(const Ctx& c) {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
     cudaGetLastError();
-    return 152 / twist_ctas(c, t);                      // no device: a 152-SM GB300
+    return 152 * (c.c64() ? 1 : 12 / t.W) / twist_ctas(c, t);   // no device: a 152-SM GB300
   }
   const void* kern = twist_function(c, t, false);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
@@ -1477,7 +1498,7 @@ int twist_concurrency(const Ctx& c) {
     if (cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg) != cudaSuccess) ncl = 0;
   }
   cudaGetLastError();
-  return ncl > 0 ? ncl : std::max(1, sms / twist_ctas(c, t));
+  return ncl > 0 ? ncl : std::max(1, sms * (c.c64() ? 1 : 12 / t.W) / twist_ctas(c, t));
 }
 
 // Geometry of k_twist_multi: the blocks beside the vectors, partial sums and compact sources
