@@ -92,8 +92,9 @@ typedef struct lsweep_params {
   double tol;         /* relative residual ||f - A u|| / ||f|| to reach (default 1e-8)*/
   void* stream;       /* cudaStream_t to issue work on; NULL = the default stream     */
   int front_kernel;   /* sweep-front kernel: 0 automatic (default: the twisted kernels where */
-                      /* they apply: 2D lines of up to about 146 nodes in complex64, 100 in */
-                      /* complex128), 1 cluster-split row slabs (any b), 2 one CTA per      */
+                      /* they apply: 2D lines of up to about 146 nodes in complex64, 108 in */
+                      /* complex128, 3D planes of up to 92), 1 cluster-split row slabs (any */
+                      /* b), 2 one CTA per                                                  */
                       /* solve streaming whole blocks, 3 the twisted kernels: a cluster per */
                       /* solve on a factor twisted at the middle line, each half            */
                       /* eliminating from one end, the symmetric block inverses stored as   */

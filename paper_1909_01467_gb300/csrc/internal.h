@@ -434,8 +434,9 @@ struct Ctx {
   std::vector<Ctx*> shifted;
   double* d_psi = nullptr;
   double2* d_win = nullptr;
-  // line vectors of the wide sweep kernel where they do not fit shared memory, one region per
-  // CTA of the largest level (allocated with the working buffers, lines_bytes)
+  // line vectors of the sweep kernels where they do not fit shared memory (wide planes; complex128
+  // twisted solves of many lines), one region per CTA of the largest level (allocated with the
+  // working buffers, lines_bytes)
   void* d_lines = nullptr;
   long long spin() const { return p.max_spin > 0 ? p.max_spin : (1LL << 30); }
   // complex64 factors and sweeps (every precision but LSWEEP_C128)
@@ -494,6 +495,7 @@ bool twist_fits(const Ctx& c);
 TileStore tile_store(const Ctx& c);
 bool twist_fused_fits(const Ctx& c);
 int twist_concurrency(const Ctx& c);
+size_t twist_lines_bytes(const Ctx& c);
 cudaError_t launch_twist(Ctx& c, const FrontArgs& a, int count, const FrontArgs* table,
                          cudaStream_t stream);
 // block sweeps over K right-hand sides (twist.cu): whether a handle can use them, the

@@ -650,10 +650,11 @@ static int wide_capacity(const Ctx& c) {
 }
 
 // bytes of line-vector scratch the plan's sweep kernels need in global memory (d_lines): the
-// wide kernel with global line vectors (NS CTAs per solve, Lmax x RB each), for the largest
-// level
+// wide kernel (NS CTAs per solve, Lmax x RB each) and complex128 twisted solves (four CTAs, their
+// half's lines and rows), for the largest level
 size_t lines_bytes(const Ctx& c) {
-  size_t need = 0;
+  // (also when the plan is set up with another kernel: lsweep_autotune may change to the twisted one)
+  size_t need = twist_lines_bytes(c);
   const size_t tasks = (size_t)std::max(1, c.max_tasks);
   Pipe pp;
   int th = 0;

@@ -45,7 +45,7 @@ struct Twist {
   TileStore ts;
   int Lh, bs;            // lines per half at most; bmax rounded up to even
   int nslot, PD;         // ring slots; steps between a copy and the L2 prefetch it issues
-  int W;                 // k_twist_rows: consumer warps
+  int W, gl;             // k_twist_rows: consumer warps; line vectors in global memory
   unsigned slot_bytes;
 };
 
@@ -755,10 +755,16 @@ k_twist(FrontArgs a_, Twist tg, const FrontArgs* __restrict__ table, int* status
 // line vectors; the owners send their entries of the next vector to the mate (st.async, two
 // barriers by step parity, re-armed one step ahead), and at the last step before the middle
 // line their part of its right-hand side to both CTAs of the other half.
+// kGlobal: the line vectors and their sources in global memory (L2-resident, a region per CTA),
+// where they do not fit beside two slots: many lines per subdomain, and the 3D planes of up to 92
+// nodes.  An owner's next entry is loaded a step ahead.  ms per application, four-CTA kernel on whole
+// blocks / cluster split on the plain factor / this: 512^2 on 2 x 8 (92-node lines, 282 of them) 23.3 /
+// 35.3 / 16.9, 1024^2 on 4 x 16 49.8 / 135 / 36.0, 24^3 on 8 x 8 beams of 81-node planes 3.8 / 7.7 /
+// 2.8; 640^2 on 8 x 8 (108-node lines) - / 46.4 / 16.0.
 constexpr int kRowsMaxCH = 32;
-template <int W, int NC>
+template <int W, int NC, bool kGlobal>
 __global__ void __launch_bounds__(W * 32 + 32, 12 / W)
-k_twist_rows(FrontArgs a, Twist tg, int* status) {
+k_twist_rows(FrontArgs a, Twist tg, double2* lines, int* status) {
   using C = double2;
   constexpr int ncons = W * 32;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -773,8 +779,9 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   const int m = twist_line(L);
   const int nf = h ? L - 1 - m : m;
   int slo, shi, nlo, nhi;
-  source_lines(g, kind, 2, slo, shi);
-  needed_lines(g, kind, 2, nlo, nhi);
+  const int dim = kGlobal ? a.dim : 2;
+  source_lines(g, kind, dim, slo, shi);
+  needed_lines(g, kind, dim, nlo, nhi);
   const int f0 = h ? min(L - 1 - shi, nf) : min(slo, nf);
   const int nsteps = nf + 1 + (h ? nhi - m : m - nlo);
   const int nit = nsteps - f0;                         // steps this CTA runs: s = f0 + it
@@ -782,7 +789,8 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   const int ka = h ? m : 0, kb = h ? L : m + 1;        // lines of this half (m in both)
   const int CH = min(kRowsMaxCH, ncons / RB), nc = (b + CH - 1) / CH;
   // shared memory: ring[nslot][slot_bytes] | full[8] | empty[8] | vbar[2] | xbar[2] | flags[4]
-  // (32-bit) | vb[2][bs] | part[32 W] | xb[bs] | H[2][bs] | V[2][Lh] | yl[Lh][RB]
+  // (32-bit) | vb[2][bs] | part[32 W] | xb[bs] | H[2][bs] | V[2][Lh] | yl[Lh][RB]; kGlobal: H, V
+  // and yl are not there, yl is this CTA's region of `lines`
   unsigned char* ring = smem_raw;
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)tg.nslot * tg.slot_bytes);
   uint64_t* empty = full + kSoloMaxSlots;
@@ -799,7 +807,7 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   C* xb = part + ncons;
   C* H = xb + bs;
   C* Vs = H + 2 * bs;
-  C* yl = Vs + 2 * tg.Lh;
+  C* yl = kGlobal ? lines + (size_t)blockIdx.x * tg.Lh * (bs / 2) : Vs + 2 * tg.Lh;
   auto line = [&](int k) { return yl + (k - ka) * nr; };
   const TileStore ts = tg.ts;
   const C* fac = reinterpret_cast<const C*>(a.fac) + g.fac_off;
@@ -845,7 +853,7 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   griddep_wait();                                       // traces of the previous level
   const Sides S(g, kind);
   const bool sweep = kind != K_RAW && kind != K_LOCAL;
-  if (sweep) {
+  if (!kGlobal && sweep) {
     side_sources<C>(a, g, kind, S, ka, kb, H, bs, Vs, tg.Lh, tid, blockDim.x);
     __syncthreads();
   }
@@ -853,9 +861,29 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
     return sweep ? side_entry<C>(S, H, bs, Vs, tg.Lh, ka, k, p)
                  : kind == K_LOCAL ? local_entry<C>(a, g, k, p) : to<C>(a.g_raw[(size_t)k * b + p]);
   };
-  for (int t = tid; t < (kb - ka) * nr; t += blockDim.x) {
-    const int kk = t / nr;
-    yl[t] = source(ka + kk, r0 + t - kk * nr);
+  // this CTA's rows of the solution: line vectors of nr entries
+  auto rows = [&](int lo, int hi) {
+    Rows R;
+    R.RB = R.ls = nr;
+    R.r0 = r0;
+    R.r1 = r0 + nr;
+    R.k0 = lo;
+    R.k1 = hi;
+    return R;
+  };
+  if constexpr (kGlobal) {
+    build_source<C>(a, g, kind, yl - (long long)ka * nr, rows(ka, kb));
+    Rows R;                                             // the first vector, every row of it
+    R.RB = R.r1 = R.ls = b;
+    R.r0 = 0;
+    R.k0 = blk(f0);
+    R.k1 = R.k0 + 1;
+    build_source<C>(a, g, kind, vb - (long long)R.k0 * b, R);
+  } else {
+    for (int t = tid; t < (kb - ka) * nr; t += blockDim.x) {
+      const int kk = t / nr;
+      yl[t] = source(ka + kk, r0 + t - kk * nr);
+    }
   }
   __syncthreads();
 
@@ -903,7 +931,7 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
       wait_middle();
     }
     for (int p = tid; p < b; p += ncons) {              // the first vector, every row of it
-      const C v = source(blk(f0), p);
+      const C v = kGlobal ? vb[p] : source(blk(f0), p);
       vb[p] = f0 >= nf ? v + xb[p] : v;
     }
     int nslot = 0;
@@ -1015,7 +1043,9 @@ k_twist_rows(FrontArgs a, Twist tg, int* status) {
   }
   cluster_arrive();                                     // the others' flags have been read
   const int o0 = h ? m + 1 : nlo, o1 = h ? nhi + 1 : m + 1;
-  if (kind != K_RAW) {
+  if (kGlobal && dim != 2) {
+    front_epilogue<C>(a, g, kind, sub, yl - (long long)ka * nr, rows(o0, o1));
+  } else if (kind != K_RAW) {
     twist_epilogue<C, 4>(
         a, g, kind, sub, yl - (long long)ka * nr - r0, nr, 0, 1, o0, o1, r0, r0 + nr,
         [&](int) { return reinterpret_cast<C*>(a.lane); },
@@ -1337,7 +1367,7 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
 
 // ---- launches ---------------------------------------------------------------------------
 // Geometry of the twisted kernels for a plan, false when they do not apply: 2D lines, and (in
-// complex64) planes of at most 92 nodes.  Tiles of 4 x 4 on one CTA per half up to 96 nodes: a
+// 3D) planes of at most 92 nodes.  Tiles of 4 x 4 on one CTA per half up to 96 nodes: a
 // 92-node line has 253 of them, two warps per scheduler, which hide one another's waits (with
 // tiles of 6 x 6, one warp per scheduler, less shared-memory traffic, an application of the
 // 1024^2 workload took 3.3 ms, with 4 x 4 2.9 ms).  Wider lines share tiles of 6 x 6 between
@@ -1355,14 +1385,14 @@ static int rows_columns(int b, int W) {
 // on whole blocks): 16 x 16 subdomains of 20-node lines 8.8 -> 2.7 (4.8), 36 nodes 13.5 -> 4.9 (9.9),
 // 52 nodes 17.8 -> 9.0 (17.9); 4 x 4 of 20 nodes 0.96 -> 0.40 (0.53), 36 nodes 1.50 -> 0.64 (1.12),
 // 52 nodes 1.96 -> 1.16 (1.95).  36 nodes with 6 warps: 6.1 and 0.86.
-static bool rows_warps(int b, int W) { return W == 12 || b <= (W == 6 ? 54 : 36); }
+static int rows_warps(int b) { return b <= 36 ? 3 : b <= 54 ? 6 : 12; }
 // tile rows at most: lines of up to 64 nodes, up to 96, wider ones on two CTAs per half
 constexpr int kGMs = 16, kGM1 = 24, kGM2 = 26;
 static bool twist_geometry(const Ctx& c, Twist& t, int& GM, int& threads, size_t& smem) {
   const bool c64 = c.c64();
   const int b = c.bmax;
   const size_t es = c.welem();
-  if (c.cube || (c.dim != 2 && !(c64 && b <= 92))) return false;
+  if (c.cube || (c.dim != 2 && b > 92)) return false;
   t.ts.NQ = !c64 || b <= 96 ? 1 : 2;
   t.ts.T = t.ts.NQ == 1 ? 4 : 6;
   t.Lh = c.Lmax - twist_line(c.Lmax);
@@ -1384,23 +1414,29 @@ static bool twist_geometry(const Ctx& c, Twist& t, int& GM, int& threads, size_t
   } else {
     GM = 0;
     if (b < 2) return false;
-    fixed += ((size_t)5 * t.bs + 2 * t.Lh + (size_t)t.Lh * ((b + 1) / 2)) * es;
-    for (int W : {3, 6, 12}) {
-      const int nc = rows_columns(b, W), per_sm = 12 / W;
-      if (!rows_warps(b, W) || nc < 1 || nc > (W == 12 ? 16 : 8)) continue;
-      const size_t limit = 228 * 1024 / per_sm - 1024, all = fixed + W * 32 * es;
+    const size_t vectors = fixed + (size_t)3 * t.bs * es;
+    const size_t lines = (2 * (size_t)t.bs + 2 * t.Lh + (size_t)t.Lh * ((b + 1) / 2)) * es;
+    t.W = rows_warps(b);
+    const int nc = rows_columns(b, t.W);
+    if (nc < 1 || nc > (t.W == 12 ? 16 : 8)) return false;
+    const size_t limit = 228 * 1024 / (12 / t.W) - 1024;
+    threads = (t.W + 1) * 32;
+    // line vectors in shared memory (2D), or, where they do not fit with as many CTAs per SM, in
+    // global memory: more solves at once are worth more (1024^2 in one row of 64 subdomains of
+    // 36-node lines, ms per application: shared memory and 12 warps 373, global and 3 warps 177)
+    for (int gl = c.dim == 2 ? 0 : 1; gl < 2; ++gl) {
+      const size_t all = vectors + (gl ? 0 : lines) + t.W * 32 * es;
       if (all + 2 * (size_t)t.slot_bytes > limit) continue;
-      t.W = W;
+      t.gl = gl;
       t.nslot = (int)std::min<size_t>(kSoloMaxSlots, (limit - all) / t.slot_bytes);
       smem = all + (size_t)t.nslot * t.slot_bytes;
-      threads = (W + 1) * 32;
       return true;
     }
     return false;
   }
   const size_t limit = 227 * 1024;
   if (fixed + 2 * (size_t)t.slot_bytes > limit) return false;
-  t.W = 0;
+  t.W = t.gl = 0;
   t.nslot = (int)std::min<size_t>(kSoloMaxSlots, (limit - fixed) / t.slot_bytes);
   smem = fixed + (size_t)t.nslot * t.slot_bytes;
   return true;
@@ -1428,12 +1464,14 @@ static TwistKernel twist_kernel(const Ctx& c, const Twist& t, bool fused) {
   if (fused) return c.bmax <= 64 ? k_twist<4, kGMs, 1, true> : k_twist<4, kGM1, 1, true>;
   return c.bmax <= 64 ? k_twist<4, kGMs, 1, false> : k_twist<4, kGM1, 1, false>;
 }
-using RowsKernel = void (*)(FrontArgs, Twist, int*);
+using RowsKernel = void (*)(FrontArgs, Twist, double2*, int*);
 static RowsKernel rows_kernel(const Ctx& c, const Twist& t) {
-  if (t.W == 3) return k_twist_rows<3, 8>;
-  if (t.W == 6) return k_twist_rows<6, 8>;
+  if (t.W == 3) return t.gl ? k_twist_rows<3, 8, true> : k_twist_rows<3, 8, false>;
+  if (t.W == 6) return t.gl ? k_twist_rows<6, 8, true> : k_twist_rows<6, 8, false>;
   const int nc = rows_columns(c.bmax, 12);
-  return nc <= 8 ? k_twist_rows<12, 8> : nc <= 12 ? k_twist_rows<12, 12> : k_twist_rows<12, 16>;
+  if (t.gl)
+    return nc <= 8 ? k_twist_rows<12, 8, true> : nc <= 12 ? k_twist_rows<12, 12, true> : k_twist_rows<12, 16, true>;
+  return nc <= 8 ? k_twist_rows<12, 8, false> : nc <= 12 ? k_twist_rows<12, 12, false> : k_twist_rows<12, 16, false>;
 }
 static const void* twist_function(const Ctx& c, const Twist& t, bool fused) {
   return c.c64() ? (const void*)twist_kernel(c, t, fused) : (const void*)rows_kernel(c, t);
@@ -1469,8 +1507,20 @@ cudaError_t launch_twist(Ctx& c, const FrontArgs& a, int count, const FrontArgs*
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   twist_config(cfg, at, twist_ctas(c, t), count, th, smem, stream, c.p.pdl != 0);
-  if (!c.c64()) return cudaLaunchKernelEx(&cfg, rows_kernel(c, t), a, t, c.d_status);
+  if (!c.c64()) {
+    if (t.gl && !c.d_lines) return cudaErrorInvalidConfiguration;
+    return cudaLaunchKernelEx(&cfg, rows_kernel(c, t), a, t, (double2*)c.d_lines, c.d_status);
+  }
   return cudaLaunchKernelEx(&cfg, twist_kernel(c, t, table != nullptr), a, t, table, c.d_status);
+}
+
+// line vectors of k_twist_rows in global memory, for the largest level
+size_t twist_lines_bytes(const Ctx& c) {
+  Twist t;
+  int GM, th;
+  size_t smem;
+  if (c.c64() || !factor_fits_smem(c) || !twist_geometry(c, t, GM, th, smem) || !t.gl) return 0;
+  return (size_t)4 * std::max(1, c.max_tasks) * t.Lh * (t.bs / 2) * sizeof(double2);
 }
 
 // lines that a fused application takes (one CTA per half)
