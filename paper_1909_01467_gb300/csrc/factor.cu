@@ -29,11 +29,14 @@ namespace lsw {
 // block leaves no room for the scratch).  Up to 96 nodes two CTAs of 256 threads share an SM, so
 // that one's tiles fill the other's steps; wider blocks are alone on theirs and take more warps,
 // as many as leave warp 0 its rows in registers (a scheduler's 16384 over its warps).
+// The column by column form also has to leave room for a second CTA (64 registers a thread; with 105
+// there was one per SM, and 16 x 16 subdomains of 36-node lines in complex128 took 15.1 ms instead
+// of 13.2).
 __host__ __device__ constexpr int simt_threads(int rpl) {
   return rpl == 0 || rpl == 4 ? 512 : rpl == 6 ? 384 : 256;
 }
 template <typename C, int RPL>
-__global__ void __launch_bounds__(simt_threads(RPL), RPL == 2 || RPL == 3 ? 2 : 1)
+__global__ void __launch_bounds__(simt_threads(RPL), RPL == 4 || RPL == 6 ? 1 : 2)
 k_factor_simt(const SubGeom* __restrict__ subs, const C* __restrict__ lcoef,
                               long long cstride, C* __restrict__ fac, int dim, TileStore ts,
                               int* __restrict__ status) {
