@@ -24,4 +24,4 @@ def test_two_ctas_share_an_sm(tmp_path):
     assert set(found) == set(FORMS)
     for form, regs in found.items():
         threads, ctas = FORMS[form]
-        assert ctas * threads * (regs + 7) // 8 * 8 <= 65536, (form, regs)
+        assert ctas * threads * ((regs + 7) // 8 * 8) <= 65536, (form, regs)
