@@ -1087,12 +1087,17 @@ __device__ inline FrontArgs rhs_args(const MultiArgs& m, int c) {
   return a;
 }
 
-// KG: right-hand sides per group at most
+// KG: right-hand sides per group at most.  OG: owners per row.  A group on lines of more than 64 nodes has
+// at least two threads per row (160 to 256 for 136 to 253 tiles), and each owns its row for every second
+// right-hand side; with one owner the others waited while it walked a round's four.  ms per block with
+// one owner -> two (the kernel on whole blocks): 1024^2 of 92-node lines, 8 right-hand sides 20.4 ->
+// 15.5 (19.6), 4 9.9 -> 8.4 (11.4); 1008^2 of 64- to 66-node lines, 8 28.3 -> 20.5 (25.1).
 template <int T, int GM, int NG, int ER, int KG>
 __global__ void __launch_bounds__(320, 1)
 k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
   using C = float2;
   constexpr int VN = T * GM, SP = part_stride(T, GM);
+  constexpr int OG = NG == 1 && KG > 1 ? 2 : 1, KO = (KG + OG - 1) / OG;   // owners per row, share
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const FrontArgs& a = ma.a;
   const int K = ma.K;
@@ -1199,8 +1204,10 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
     const bool worker = worker_tile<1>(gt, G, 0, I, J);
     const unsigned unit = (unsigned)tile_count(G, 1, 0) * 16;
     const unsigned tile_off = worker ? (unsigned)gt * 16 : 0;
-    const bool owner = gt < b;
-    const int OI = owner ? gt / T : 0, oi = owner ? gt - OI * T : 0;
+    const int og = OG == 1 ? 0 : gt / (gth / OG);         // owner: row ot, right-hand sides og + OG i
+    const int ot = OG == 1 ? gt : gt - og * (gth / OG);
+    const bool owner = ot < b;
+    const int OI = owner ? ot / T : 0, oi = owner ? ot - OI * T : 0;
     const int cpl_off = part_cpl(b, ts, 0);
     int doff[T];
 #pragma unroll
@@ -1215,21 +1222,22 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
       return to<C>(ma.rin[c][(size_t)(g.gy0 + k) * a.Ne + g.gx0 + p]);
     };
     auto send_middle = [&](int c, C v) {
-      st_async(mapa(smem_u32(xb + c * bs + gt), peer), v, rbar);
+      st_async(mapa(smem_u32(xb + c * bs + ot), peer), v, rbar);
       flags[0] = 1;
     };
     // operands of step it: the next line's source (forward), or y_k (backward: stored by this
     // thread at least two steps before, or zero on a line whose forward step was skipped)
-    C An[KG];
+    C An[KO];
     auto fetch = [&](int it) {
       const int s = f0 + it, k = blk(s);
       const bool seen = (h ? L - 1 - k : k) >= f0;
 #pragma unroll
-      for (int e = 0; e < KG; ++e) {
-        An[e] = czero<C>();
+      for (int i = 0; i < KO; ++i) {
+        const int e = og + OG * i;
+        An[i] = czero<C>();
         if (owner && e < kg && it < nit) {
-          if (s < nf) An[e] = source(rhs(e), h ? k - 1 : k + 1, gt);
-          else if (s > nf && seen) An[e] = __ldcg(yl + (size_t)k * LS + rhs(e) * b + gt);
+          if (s < nf) An[i] = source(rhs(e), h ? k - 1 : k + 1, ot);
+          else if (s > nf && seen) An[i] = __ldcg(yl + (size_t)k * LS + rhs(e) * b + ot);
         }
       }
     };
@@ -1237,14 +1245,14 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
       const int k = blk(f0);
       if (f0 >= nf) {
         // the middle line comes first (see k_twist)
-        for (int e = 0; e < kg; ++e) send_middle(rhs(e), czero<C>());
+        for (int e = og; e < kg; e += OG) send_middle(rhs(e), czero<C>());
         mbar_wait<true>(xbar, 0, status, timed_out, a.spin);
       }
-      for (int e = 0; e < kg; ++e) {
+      for (int e = og; e < kg; e += OG) {
         const int c = rhs(e);
-        C v = source(c, k, gt);
-        if (f0 >= nf) v = v + xb[c * bs + gt];
-        vb[c * 2 * VN + gt] = v;
+        C v = source(c, k, ot);
+        if (f0 >= nf) v = v + xb[c * bs + ot];
+        vb[c * 2 * VN + ot] = v;
       }
     }
     fetch(0);
@@ -1252,7 +1260,7 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
     uint32_t phase = 0;
     C D[T * T], dr[T];
     auto ready = [&]() { mbar_wait<false>(&full[nslot], phase, status, timed_out, a.spin); };
-    const int lrow = owner ? gt : 0;
+    const int lrow = owner ? ot : 0;
     ready();
 #pragma unroll
     for (int i = 0; i + 2 < T; i += 2) load_rows<T>(D, ring + tile_off, unit, i);
@@ -1269,9 +1277,9 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
       const C cc = sl[cpl_off + ((s < nf) == (h != 0) ? (b + 1) & ~1 : 0) + lrow];
 #pragma unroll
       for (int j = 0; j < T; ++j) dr[j] = sl[doff[j]];
-      C Ac[KG];
+      C Ac[KO];
 #pragma unroll
-      for (int e = 0; e < KG; ++e) Ac[e] = An[e];
+      for (int i = 0; i < KO; ++i) Ac[i] = An[i];
       fetch(it + 1);
       auto tile = [&](int e, int pb, auto refill) {
         const C* v = vb + rhs(e) * 2 * VN + (it & 1) * VN;
@@ -1303,30 +1311,31 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
         consumer_sync(ncons);                           // the partial sums are there
         if (owner) {
 #pragma unroll
-          for (int u = 0; u < ER; ++u) {
-            const int e = e0 + u;
-            if (e >= KG || e >= e1) continue;
-            const int c = rhs(e);
+          for (int i = 0; i < ER / OG; ++i) {
+            const int at = e0 / OG + i;                   // (its place in Ac)
+            const int e = e0 + og + OG * i;
+            if (at >= KO || e >= e1) continue;
+            const int c = rhs(e), u = e - e0;
             C vO[T], dA = czero<C>(), dB = dA;
             load_run<T>(vb + c * 2 * VN + (it & 1) * VN + OI * T, vO);
 #pragma unroll
             for (int j = 0; j < T; ++j) mac(dr[j], vO[j], dA, dB);
-            const C sum = row_sum<T, GM, 1>(part + (u * NG + grp) * GM * SP + gt, G, OI, 0,
+            const C sum = row_sum<T, GM, 1>(part + (u * NG + grp) * GM * SP + ot, G, OI, 0,
                                             mk(dA.x - dA.y, dB.x + dB.y));
-            C* yk = yl + (size_t)k * LS + c * b + gt;
+            C* yk = yl + (size_t)k * LS + c * b + ot;
             C nv;
             if (s < nf) {
               *yk = sum;                                // y_k (z_k)
               const C t = cmul(cc, sum);
-              nv = Ac[e] - t;
+              nv = Ac[at] - t;
               // every owner sends, timed out or not: all rows or none
               if (mid) send_middle(c, mk(-t.x, -t.y));
             } else {
-              const C x = s == nf ? sum : Ac[e] - sum;
+              const C x = s == nf ? sum : Ac[at] - sum;
               *yk = x;
               nv = cmul(cc, x);
             }
-            vb[c * 2 * VN + ((it + 1) & 1) * VN + gt] = nv;
+            vb[c * 2 * VN + ((it + 1) & 1) * VN + ot] = nv;
           }
         }
       }
@@ -1337,10 +1346,10 @@ k_twist_multi(const __grid_constant__ MultiArgs ma, Twist tg, int* status) {
       if (owner && mid && kg > 0) {
         // add the other half's parts of line m's right-hand side
         mbar_wait<true>(xbar, 0, status, timed_out, a.spin);
-        for (int e = 0; e < kg; ++e) {
+        for (int e = og; e < kg; e += OG) {
           const int c = rhs(e);
-          C* nv = vb + c * 2 * VN + ((it + 1) & 1) * VN + gt;
-          *nv = *nv + xb[c * bs + gt];
+          C* nv = vb + c * 2 * VN + ((it + 1) & 1) * VN + ot;
+          *nv = *nv + xb[c * bs + ot];
         }
       }
       if (timed_out) stop_at(stop, it);
