@@ -441,7 +441,8 @@ int build_plan(Ctx* c) {
     }
   }
   // plans whose sweeps stream half rows store those, the others whole blocks or triangles
-  c->half_rows = lsw::uses_wide(*c);
+  c->wide = lsw::uses_wide(*c);
+  c->half_rows = c->wide && !lsw::wide_whole(*c);
   const lsw::TileStore ts = lsw::twist_fits(*c) ? lsw::tile_store(*c) : lsw::TileStore{0, 1};
   for (auto& g : c->subs) {
     if (c->half_rows) g.bs = lsw::half_stride(g.b);
@@ -1109,6 +1110,7 @@ int lsweep_clone(lsweep_handle h, void* stream, lsweep_handle* out) {
   c->alpha_entries = p->alpha_entries; c->Lmax = p->Lmax; c->bmax = p->bmax;
   c->bpmax = p->bpmax; c->trace_W = p->trace_W; c->fac_elems = p->fac_elems;
   c->pz = p->pz; c->cube = p->cube; c->n_trace_arr = p->n_trace_arr;
+  c->wide = p->wide;
   c->half_rows = p->half_rows;
   c->node_elems = p->node_elems;
   for (int f = 0; f < 3; ++f) {
@@ -1347,7 +1349,7 @@ std::vector<TuneCand> tune_candidates(Ctx* c) {
   // the storage laid out at setup (half rows or whole blocks) stays
   cands.erase(std::remove_if(cands.begin(), cands.end(), [&](const TuneCand& x) {
                 c->p.front_kernel = x.kernel;
-                return lsw::uses_wide(*c) != c->half_rows;
+                return lsw::uses_wide(*c) != c->wide;
               }),
               cands.end());
   c->p = saved;

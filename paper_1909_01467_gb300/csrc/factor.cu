@@ -590,7 +590,9 @@ static size_t simt_smem(const Ctx& c, int rpl) {
 bool factor_fits_smem(const Ctx& c) { return simt_smem(c, 0) <= 227 * 1024; }
 
 cudaError_t launch_factor(Ctx& c) {
-  if (c.half_rows || !factor_fits_smem(c))
+  // (planes of the wide sweep kernel that would fit are inverted faster in panels: complex128 lines of
+  // 112 nodes, 462 of them on 2 x 10 subdomains, 1270 -> 860 ms)
+  if (c.wide || !factor_fits_smem(c))
     return c.c64() ? launch_factor_wide<float2>(c) : launch_factor_wide<double2>(c);
   const TileStore ts = c.fac_twisted ? tile_store(c) : TileStore{0, 1};
   auto launch = [&](auto kern, auto zero, int rpl) {

@@ -347,7 +347,8 @@ struct Ctx {
   bool cube = false;
   std::vector<AxisBlock> zb;
   int n_trace_arr = N_TRACE_ARR;
-  bool half_rows = false;       // the sweeps run on k_front_wide: blocks stored as half rows
+  bool wide = false;            // the sweeps run on k_front_wide
+  bool half_rows = false;       // and its blocks are stored as half rows
   std::vector<SubGeom> subs;
   std::vector<AlphaSeg> segs;   // PML tables: global, then one per x, y (and z) block
   int alpha_entries = 0;
@@ -508,6 +509,8 @@ cudaError_t launch_front_multi(Ctx& c, int li, int K, Ctx* const* rhs, const dou
 void set_global_error(const std::string& msg);
 bool front_pipeline_fits(const Ctx& c);
 bool uses_wide(const Ctx& c);
+// whether that plan's blocks stay whole
+bool wide_whole(const Ctx& c);
 // bytes of global line-vector scratch (d_lines) the plan's sweep kernels need (0: none)
 size_t lines_bytes(const Ctx& c);
 // true when lsweep_factor should store twisted factors: sweep-front kernel 0 (automatic) or 3,

@@ -583,7 +583,7 @@ static cudaError_t launch_front_t(Ctx& c, const Task* tasks, int off, int count,
   Pipe pp;
   int th = 0;
   size_t smem = 0;
-  if (c.half_rows) return launch_front_wide<C>(c, a, count);
+  if (c.wide) return launch_front_wide<C>(c, a, count);
   if (!choose_pipe<C>(c, count, pp, th, smem)) return cudaErrorInvalidConfiguration;
   auto kern = c.cube ? k_front<C, true> : k_front<C, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -653,8 +653,8 @@ static int wide_capacity(const Ctx& c) {
 // wide kernel (NS CTAs per solve, Lmax x RB each) and complex128 twisted solves (four CTAs, their
 // half's lines and rows), for the largest level
 size_t lines_bytes(const Ctx& c) {
-  // (also when the plan is set up with another kernel: lsweep_autotune may change to the twisted one)
-  size_t need = twist_lines_bytes(c);
+  // (also when the plan is set up with another kernel that lsweep_autotune may change from)
+  size_t need = c.wide ? 0 : twist_lines_bytes(c);
   const size_t tasks = (size_t)std::max(1, c.max_tasks);
   Pipe pp;
   int th = 0;
@@ -683,6 +683,8 @@ bool uses_wide(const Ctx& c) {
   }
   return !choose_pipe<double2>(c, 1, pp, th, smem);
 }
+
+bool wide_whole(const Ctx& c) { return wide_whole_rows(c); }
 
 bool front_pipeline_fits(const Ctx& c) {
   Pipe pp;

@@ -31,6 +31,7 @@ namespace lsw {
 // receiver's mbarrier); the row owners add them to their row sums in a fixed order, update the
 // line vectors, and each CTA sends its rows of the next right-hand vector to the others as one
 // bulk copy each.
+// Blocks that stay whole (NW = 0, wide_whole_rows) take the same path without column sums.
 // Measured against whole rows, one application: 96^3 on 6 x 6 beams (planes of up to 1024 nodes)
 // 66.1 -> 49.1 ms, 48^3 on 3 x 3 x 3 boxes 21.9 -> 18.4 ms.  A step of 16 chunks takes 24.6 k
 // clocks, 20.1 k of them in the chunks (19.2 k at the measured copy bandwidth with 120 SMs
@@ -91,7 +92,8 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
   const Task task = a.tasks[a.task_off + blockIdx.x / NS];
   const int sub = task.sub, kind = task.kind;
   const SubGeom g = a.subs[sub];
-  const int b = g.b, hp = half_row(b), hw = b / 2, L = g.L;
+  constexpr bool kHalf = NW > 0;                        // blocks stored as half rows, or whole
+  const int b = g.b, hp = kHalf ? half_row(b) : g.bp, hw = b / 2, L = g.L;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   constexpr int CH = 8, HV = wide_halves<C>();          // rows per chunk, warps per row
   constexpr int ncw = CH * HV, ncons = ncw * 32;         // consumer warps and threads
@@ -106,7 +108,7 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
   // CTAs that have rows (a small box may leave the last ones without: they take no part in the
   // exchanges, so nothing is sent to them either)
   const int NA = (b + RB - 1) / RB;
-  const int ncol = nr > 0 ? nr + hw : 0;                 // columns this CTA's rows touch
+  const int ncol = kHalf && nr > 0 ? nr + hw : 0;        // columns this CTA's rows touch
   // shared memory: ring | full[8] | empty[8] | vbar[2] | rbar (+pad) | ysum[HV][RB] | own[RB] |
   // recv[NS][RB] | vk[2][bmax + 2] | part[ncw][PW] | yl[Lmax][RB]
   unsigned char* ring = smem_raw;
@@ -117,10 +119,10 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
   C* ysum = reinterpret_cast<C*>(vbar + 8);
   C* own = ysum + HV * wp.RB;
   C* recv = own + wp.RB;
-  C* vk = recv + NS * wp.RB;
+  C* vk = kHalf ? recv + NS * wp.RB : own;               // (whole rows: no column sums)
   const int vs = (wp.bmax + 3) & ~1;                     // (a rounded copy may pass row b)
   C* part = vk + 2 * vs;
-  const int PW = 32 * ((wp.RB + 31) / 32 + NW);          // columns of a warp's sums
+  const int PW = kHalf ? 32 * ((wp.RB + 31) / 32 + NW) : 0;   // columns of a warp's sums
   // line vectors: shared memory, or (when they do not fit beside the ring: smaller clusters
   // of more rows per CTA) one global region per CTA; a thread then owns at most one row and
   // loads its next line entry at the start of each step
@@ -147,7 +149,7 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
     return n;
   };
   uint32_t recv_bytes = 0;
-  for (int q = 0; q < NS; ++q) recv_bytes += (uint32_t)(overlap(q) * (int)sizeof(C));
+  for (int q = 0; kHalf && q < NS; ++q) recv_bytes += (uint32_t)(overlap(q) * (int)sizeof(C));
   bool timed_out = false;
   auto blk = [&](int s) { return s < L ? s : 2 * L - 2 - s; };
   const int total = nsteps * nch;                        // chunk copies of the whole solve
@@ -189,10 +191,10 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
     if (NS > 1) {
       mbar_expect_tx(&vbar[0], peer_bytes);
       if (nsteps > 1) mbar_expect_tx(&vbar[1], peer_bytes);
-      mbar_expect_tx(rbar, recv_bytes);
+      if (kHalf) mbar_expect_tx(rbar, recv_bytes);
     }
   }
-  for (int t = tid; t < NS * wp.RB; t += blockDim.x) recv[t] = czero<C>();
+  for (int t = tid; kHalf && t < NS * wp.RB; t += blockDim.x) recv[t] = czero<C>();
   if (NS > 1) cluster_sync_all();
   else __syncthreads();
   const bool producer = tid == ncons;                    // lane 0 of the last warp
@@ -247,8 +249,8 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
       // RB <= ncons)
       C line_pre = czero<C>(), cpl_pre = line_pre;
       // couplings l_k, then l_{k-1}: the one towards the line of the next vector
-      const C* cpl = fac + (size_t)k * g.bs + half_cpl(b) +
-                     (fwd && k + 1 < L ? 0 : (b + 1) & ~1) + R.r0;
+      const C* cpl = fac + (size_t)k * g.bs + b * hp +
+                     (fwd && k + 1 < L ? 0 : kHalf ? (b + 1) & ~1 : hp) + R.r0;
       if (tid < nr) {
         cpl_pre = cpl[tid];
         if (wp.lines) {
@@ -274,7 +276,7 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
         cnext = cnext >= b ? cnext - b : cnext;
         return x;
       };
-      C vc[NW], yc[NW];
+      C vc[kHalf ? NW : 1], yc[kHalf ? NW : 1];
 #pragma unroll
       for (int u = 0; u < NW; ++u) {
         vc[u] = entry();
@@ -295,6 +297,19 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
           const int j0 = first - rr, last = rl < nr ? hw - j0 : -1;
           const uint32_t row = ring_at + (uint32_t)slot * wp.slot_bytes +
                                (uint32_t)((rw * hp + j0) * (int)sizeof(C));
+          if constexpr (!kHalf) {
+            // the whole row, columns 32 apart, in four sums
+            const C* d = reinterpret_cast<const C*>(ring + (size_t)slot * wp.slot_bytes) + rw * hp;
+            C p[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) p[u] = czero<C>();
+            if (rl < nr)
+              for (int c0 = lane; c0 < b; c0 += 128)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  if (c0 + 32 * u < b) p[u] = cfma(d[c0 + 32 * u], v[c0 + 32 * u], p[u]);
+            acc[q] = (p[0] + p[1]) + (p[2] + p[3]);
+          }
           const C vr = v[min(R.r0 + rl, b - 1)];
           // n groups of the window: the last one holds no entry of the first rows of a group of 32,
           // which complex128, bound by these multiply-adds, leaves out (a body of its own: where the
@@ -315,8 +330,10 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
             }
             acc[q] = A + B;
           };
-          if (HV == 1 && 32 * (NW - 1) > rr + hw) products(std::integral_constant<int, NW - 1>());
-          else products(std::integral_constant<int, NW>());
+          if constexpr (kHalf) {
+            if (HV == 1 && 32 * (NW - 1) > rr + hw) products(std::integral_constant<int, NW - 1>());
+            else products(std::integral_constant<int, NW>());
+          }
           __syncwarp();
           // (a warp whose wait gave up never releases the slot: the copy may still be landing)
           if (lane == 0 && !timed_out) mbar_arrive(&empty[slot]);
@@ -328,56 +345,63 @@ k_front_wide(FrontArgs a, Wide wp, int* status) {
         const C sum = warp_rows4<C>(acc, lane);          // lane 8 q: the row of chunk q
         const int rl = 32 * g32 + lane + rw;
         if ((lane & 7) == 0 && rl < nr) ysum[w / CH * wp.RB + rl] = sum;
-        mine[32 * g32] = yc[0];                          // the window moves on
+        if constexpr (kHalf) {
+          mine[32 * g32] = yc[0];                        // the window moves on
 #pragma unroll
-        for (int u = 0; u + 1 < NW; ++u) {
-          vc[u] = vc[u + 1];
-          yc[u] = yc[u + 1];
+          for (int u = 0; u + 1 < NW; ++u) {
+            vc[u] = vc[u + 1];
+            yc[u] = yc[u + 1];
+          }
+          vc[NW - 1] = entry();
+          yc[NW - 1] = czero<C>();
         }
-        vc[NW - 1] = entry();
-        yc[NW - 1] = czero<C>();
       }
 #pragma unroll
       for (int u = 0; u < NW; ++u) mine[32 * ((nr + 31) / 32 + u)] = yc[u];
       consumer_sync(ncons);                              // row and column sums are complete
+      if constexpr (kHalf) {
 #pragma unroll
-      for (int i = 0; i < kMyCols; ++i) {
-        const int cidx = tid + i * ncons;
-        if (cidx >= ncol) break;
-        C sum = czero<C>();
+        for (int i = 0; i < kMyCols; ++i) {
+          const int cidx = tid + i * ncons;
+          if (cidx >= ncol) break;
+          C sum = czero<C>();
 #pragma unroll
-        for (int hv = 0; hv < HV; ++hv) {
-          const int rel = cidx - hv * 32 * NW;           // in the windows of these warps
-          if (rel < 0 || rel >= 32 * ((nr + 31) / 32 + NW)) continue;
-          const C* p = part + (size_t)hv * CH * PW + rel;
-          C s0 = czero<C>(), s1 = czero<C>();
+          for (int hv = 0; hv < HV; ++hv) {
+            const int rel = cidx - hv * 32 * NW;           // in the windows of these warps
+            if (rel < 0 || rel >= 32 * ((nr + 31) / 32 + NW)) continue;
+            const C* p = part + (size_t)hv * CH * PW + rel;
+            C s0 = czero<C>(), s1 = czero<C>();
 #pragma unroll
-          for (int ww = 0; ww < CH; ww += 2) {
-            s0 = s0 + p[ww * PW];
-            s1 = s1 + p[(ww + 1) * PW];
+            for (int ww = 0; ww < CH; ww += 2) {
+              s0 = s0 + p[ww * PW];
+              s1 = s1 + p[(ww + 1) * PW];
+            }
+            sum = sum + (s0 + s1);
           }
-          sum = sum + (s0 + s1);
+          if (cidx < nr) {
+            own[cidx] = sum;
+          } else {
+            int c = R.r0 + cidx;
+            while (c >= b) c -= b;
+            const int q = c / RB;
+            C* dst = recv + rank * wp.RB + c - q * RB;
+            if (q == rank) *dst = sum;
+            else st_async(mapa(smem_u32(dst), (uint32_t)q), sum, mapa(smem_u32(rbar), (uint32_t)q));
+          }
         }
-        if (cidx < nr) {
-          own[cidx] = sum;
-        } else {
-          int c = R.r0 + cidx;
-          while (c >= b) c -= b;
-          const int q = c / RB;
-          C* dst = recv + rank * wp.RB + c - q * RB;
-          if (q == rank) *dst = sum;
-          else st_async(mapa(smem_u32(dst), (uint32_t)q), sum, mapa(smem_u32(rbar), (uint32_t)q));
-        }
+        if (NS > 1 && tid < nr) mbar_wait(rbar, (uint32_t)(s & 1), status, timed_out);
+        consumer_sync(ncons);
+        // the next step's column sums are sent after the vector that this CTA's rows are part
+        // of, so the barrier is re-armed before any can arrive
+        if (NS > 1 && tid == 0 && s + 1 < nsteps) mbar_expect_tx(rbar, recv_bytes);
       }
-      if (NS > 1 && tid < nr) mbar_wait(rbar, (uint32_t)(s & 1), status, timed_out);
-      consumer_sync(ncons);
-      // the next step's column sums are sent after the vector that this CTA's rows are part
-      // of, so the barrier is re-armed before any can arrive
-      if (NS > 1 && tid == 0 && s + 1 < nsteps) mbar_expect_tx(rbar, recv_bytes);
       for (int rl = tid; rl < nr; rl += ncons) {
-        C sum = ysum[rl] + own[rl];
-        if (HV == 2) sum = sum + ysum[wp.RB + rl];
-        for (int q = 0; q < NA; ++q) sum = sum + recv[q * wp.RB + rl];
+        C sum = ysum[rl];
+        if constexpr (kHalf) {
+          sum = sum + own[rl];
+          if (HV == 2) sum = sum + ysum[wp.RB + rl];
+          for (int q = 0; q < NA; ++q) sum = sum + recv[q * wp.RB + rl];
+        }
         const C cc = rl == tid ? cpl_pre : cpl[rl];
         C nv = czero<C>(), ynew;
         if (fwd) {

@@ -46,6 +46,14 @@ inline int wide_window(int nw, bool cube) {
   return nw <= 3 && !cube ? 3 : nw <= 5 ? 5 : nw <= 9 ? 9 : 14;
 }
 
+// Blocks stored and streamed whole (NW = 0): complex128 lines of up to 128 nodes.  A step is then two
+// chunks of rows per CTA (clusters of 8), a half row's 58 to 65 entries take up to three groups of its
+// window (24 multiply-adds a lane where the whole row has 16), and a step of so few rows does not pay
+// for the exchange of column sums.  ms per application, half -> whole rows: 114 nodes (2 x 10
+// subdomains) 85.7 -> 64.5, 128 nodes (2 x 8) 72.7 -> 51.1; from 129 nodes on, with a third chunk, half
+// rows are faster: 130 nodes (2 x 7) 63.8 against 73.4, 140 nodes (2 x 8) 101 against 127.
+inline bool wide_whole_rows(const Ctx& c) { return !c.c64() && c.dim == 2 && c.bmax <= 128; }
+
 // Geometry of k_front_wide: NS CTAs per solve (the smallest of 2, 4, 8, 16 whose rows and line
 // vectors fit beside a ring of at least 2 chunks of 8 whole rows: the planes that fit so were
 // taken before the rows were halved, and the ring has twice the depth for it).  The window of
@@ -59,22 +67,26 @@ inline bool choose_wide(const Ctx& c, Wide& wp, size_t& smem) {
   wp.bmax = c.bmax;
   wp.gl = 0;
   wp.lines = nullptr;
-  wp.slot_bytes = (unsigned)(((size_t)wp.CH * half_row(c.bmax) * sizeof(C) + 127) / 128 * 128);
   const size_t whole = ((size_t)wp.CH * c.bpmax * sizeof(C) + 127) / 128 * 128;
+  const bool half = !wide_whole_rows(c);
+  wp.slot_bytes = half ? (unsigned)(((size_t)wp.CH * half_row(c.bmax) * sizeof(C) + 127) / 128 * 128)
+                       : (unsigned)whole;
   constexpr int HV = wide_halves<C>(), ncons = 8 * HV * 32;
   for (int ns : {2, 4, 8, 16}) {
     const int rb = ((c.bmax + ns - 1) / ns + 1) / 2 * 2;
     // groups of 32 columns a row's 32-row window spans, per warp of the row
     const int nw = (c.bmax / 2 / 32 + 2 + HV - 1) / HV;
-    wp.NW = wide_window<C>(nw, c.cube);
+    wp.NW = half ? wide_window<C>(nw, c.cube) : 0;
     // (a thread completes at most wide_my_cols of the columns)
     const int cols = HV == 2 ? 32 * (wp.NW * HV + 8) : wide_my_cols<C>(wp.NW) * ncons;
-    if (nw > wp.NW || rb + c.bmax / 2 > cols) continue;
+    if (half && (nw > wp.NW || rb + c.bmax / 2 > cols)) continue;
     const size_t lines = (size_t)c.Lmax * rb * sizeof(C);
     const size_t old_vec = 24 * sizeof(uint64_t) + ((size_t)rb + 2 * (size_t)c.bmax) * sizeof(C);
     const size_t vec = 24 * sizeof(uint64_t) +
-                       ((size_t)(1 + HV + ns) * rb + 2 * (size_t)(c.bmax + 3) +
-                        (size_t)wp.CH * HV * 32 * ((rb + 31) / 32 + wp.NW)) * sizeof(C);
+                       ((size_t)HV * rb + 2 * (size_t)(c.bmax + 3) +
+                        (half ? (size_t)(1 + ns) * rb +
+                                    (size_t)wp.CH * HV * 32 * ((rb + 31) / 32 + wp.NW)
+                              : 0)) * sizeof(C);
     // the line vectors in shared memory, or in global memory (the handle's d_lines): clusters
     // of 8 CTAs whose rows the consumer threads cover one each (two clusters per GPC instead
     // of one of 16; fewer CTAs per solve would lengthen each solve's dependent chain)
