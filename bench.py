@@ -72,9 +72,8 @@ def parse():
     ap.add_argument("--skip-c128", action="store_true",
                     help="do not time the complex128 form beside the mixed one")
     ap.add_argument("--front-kernel", type=int, default=0, choices=[0, 1, 2, 3],
-                    help="sweep-front kernel of the complex64 form: 0 automatic (3), 1 cluster "
-                         "split, 2 one CTA per solve, 3 two CTAs per solve on the twisted "
-                         "factor")
+                    help="sweep-front kernel of the complex64 form: 0 automatic (the twisted "
+                         "kernels), 1 cluster split, 2 one CTA per solve, 3 the twisted kernels")
     ap.add_argument("--no-pdl", action="store_true",
                     help="launch the sweep levels in plain stream order (no programmatic "
                          "dependent launch)")
@@ -429,8 +428,8 @@ def run_ours(args):
             c128_roof = {"bound": "alu", "achieved": ach, "peak": FP64_TFLOPS, "unit": "TFLOP/s",
                          "frac": ach / FP64_TFLOPS, "traffic": None,
                          "kernel": "k_twist_rows (four CTAs per local solve on the "
-                                   "twisted factor, line vectors in global memory): FP64 "
-                                   "block-vector products",
+                                   "twisted factor, stored as triangles): FP64 block-vector "
+                                   "products",
                          "peak_source": "nominal GB300 FP64 rate (no measured FP64 peak)",
                          "hbm_gbs": gbs, "hbm_frac": gbs / peak_hbm,
                          "front_ms_per_step": pc.front_ms,

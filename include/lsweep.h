@@ -94,15 +94,15 @@ typedef struct lsweep_params {
   int front_kernel;   /* sweep-front kernel: 0 automatic (default: the twisted kernels where */
                       /* they apply: 2D lines of up to about 146 nodes in complex64, 108 in */
                       /* complex128, 3D planes of up to 92), 1 cluster-split row slabs (any */
-                      /* b), 2 one CTA per                                                  */
-                      /* solve streaming whole blocks, 3 the twisted kernels: a cluster per */
-                      /* solve on a factor twisted at the middle line, each half            */
-                      /* eliminating from one end, the symmetric block inverses stored as   */
-                      /* triangles (2 and 3: complex64, line width b <= 92 only)            */
+                      /* b), 2 one CTA per solve streaming whole blocks, 3 the twisted      */
+                      /* kernels: a cluster per solve on a factor twisted at the middle     */
+                      /* line, each half eliminating from one end, the symmetric block      */
+                      /* inverses stored as triangles (2 and 3: complex64, line width       */
+                      /* b <= 92 only)                                                      */
   int prefetch_steps; /* kernels 2, 3: steps of bulk L2 prefetch ahead of the block      */
                       /* stream; planes too wide for a row slab per ring slot (3D): row  */
                       /* chunks between a ring copy and the L2 prefetch it issues        */
-                      /* (default 3);                                                    */
+                      /* (default 6);                                                    */
                       /* 0..16; -1 selects the default (0)                              */
   int schedule;       /* order of the local solves of one application: 0 (default)     */
                       /* dependency levels (same operations per trace and lane as the   */
@@ -391,7 +391,7 @@ int lsweep_ext_size(lsweep_handle h, int64_t* n_ext);
  * lines where the right-hand side is zero: one-CTA and twisted kernels; backward past the last
  * line that is read: twisted kernels).  Twisted factors store and stream the triangle of each
  * block, (b + 1) / (2 b) of this, and the kernel of planes too wide for a row slab half rows, as
- * many bytes (lsweep_profile.front_bytes).  A plan that the twisted kernels take holds
+ * many bytes (lsweep_profile.front_bytes; complex128 lines of up to 128 nodes: whole blocks).  A plan that the twisted kernels take holds
  * room for whole blocks as well, which lsweep_autotune may change to: its allocation is the larger
  * of the two forms, not the stored bytes.  Host outputs. */
 int lsweep_factor_bytes(lsweep_handle h, int64_t* stored, int64_t* per_apply);

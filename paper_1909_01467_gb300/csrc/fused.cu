@@ -105,8 +105,8 @@ struct Fused {
           front_form(r0) == 0 || (c->twisted() && !twist_fused_fits(*c))) {
         msg = "problems need complex64 factors, no windows, no cube CDD, the same line width, "
               "padded width "
-              "and line count, and the same sweep-front form (two CTAs per solve on twisted "
-              "factors, or one CTA per solve)";
+              "and line count, and the same sweep-front form (twisted factors, or one CTA per "
+              "solve)";
         return LSWEEP_EINVAL;
       }
     }

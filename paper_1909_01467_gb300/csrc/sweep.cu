@@ -21,8 +21,10 @@
 // products that are summed per row through shared memory; the row's senders then write
 // the next right-hand-side entry to this CTA's vector and send it to the other CTAs of the
 // cluster with st.async remote stores that complete on the receiver's mbarrier
-// (distributed shared memory), so a step needs no cluster-wide barrier.  The line vectors (source, y, x) and the line couplings
-// of the CTA's rows stay in shared memory for the whole solve.
+// (distributed shared memory), so a step needs no cluster-wide barrier.  The line vectors
+// (source, y, x) and the line couplings of the CTA's rows stay in shared memory for the whole
+// solve.  The kernels on twisted factors are in twist.cu, the one for planes too wide for a row
+// slab per slot in wide.cuh.
 #include <algorithm>
 #include <type_traits>
 

@@ -14,9 +14,9 @@ namespace lsw {
 // streams its factor from HBM twice, so its bytes are what the solve costs.  The block
 // inverses are symmetric: of each unordered pair of entries one is stored, row r holding the
 // columns r, r + 1, .., r + b / 2 (mod b) (half_row entries; for even b the antipodal pair has a
-// place in both rows, zero in the later one).  All rows have the same length, so any range of rows is contiguous and
-// as long as any other of its size.  An entry d = D[r][c] is used twice: d v_c for row r's
-// sum, and d v_r for row c's.
+// place in both rows, zero in the later one).  All rows have the same length, so any range of rows
+// is contiguous and as long as any other of its size.  An entry d = D[r][c] is used twice: d v_c
+// for row r's sum, and d v_r for row c's.
 // A solve runs on a cluster of NS CTAs (up to 16); CTA q owns rows [q RB, (q+1) RB) of every
 // block, and its producer warp streams them in chunks of CH rows through a ring of NSLOT
 // shared-memory slots (one bulk copy per chunk).  Two warps (complex128, bound by the FP64

@@ -1,5 +1,5 @@
-"""complex128 twisted solves whose line vectors do not fit shared memory: subdomains of many lines, lines
-of 101 to 108 nodes, and 3D planes of up to 92 nodes (all of whose sources are built in global memory).
+"""complex128 twisted solves whose line vectors do not fit shared memory, and the widest that do:
+subdomains of many lines, lines of 99 to 108 nodes, and 3D planes of up to 92 nodes (all of whose sources are built in global memory).
 
 Each plan stores fewer factor bytes than for the cluster split (it is twisted: triangles instead of
 whole blocks); its applications match the oracle's within 1e-10, directly and
@@ -44,9 +44,10 @@ def setup(L, dim, n, npml, q, r, **kw):
     return Problem(m, omega, npml), h
 
 
-# lines x nodes: 228 x 90 (12 warps), 176 x 36 (3 warps), 312 x 52 (6 warps), 108 x 108; planes of 36
-# to 81 nodes
+# lines x nodes: 228 x 90 (12 warps), 176 x 36 (3 warps), 312 x 52 (6 warps), 108 x 108; in shared
+# memory still 99 x 99 and 100 x 100 (the widest); 198 x 92 just past it; planes of 36 to 81 nodes
 PLANS = [(2, 420, 8, 2, 6), (2, 160, 8, 1, 10), (2, 288, 12, 1, 12), (2, 240, 12, 3, 3),
+         (2, 213, 12, 3, 3), (2, 216, 12, 3, 3), (2, 360, 8, 2, 5),
          (3, 9, 1, 3, 3), (3, 6, 1, 2, 2), (3, 5, 2, 1, 1)]
 
 
