@@ -37,12 +37,6 @@ if ROOT not in sys.path:
 METRIC = "solve unknowns/s at rel. residual 1e-8 (mixed vs complex128); sweep HBM GB/s"
 WORKLOAD = "smooth2d n=1024 npml=12 cdd=16x16 (64^2 subdomains) 4 sources tol=1e-8"
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one sweep-front launch of
-# the default workload (two- and four-CTA kernels on the twisted factor, capped dependency
-# levels), mean over the launches of one ncu capture.  Reported only while the kernel source
-# is the one it was measured on.
-FRONT_TRAFFIC = {"sweep_cu_sha256": "928d0015646443eee12de1845b4b4d81e2015d7ad36a9cc607b57e304d3dcfcd",
-                 "bytes_per_launch": 589.0e6, "n": 1024, "front_kernels": (0,)}
 # FP64 oracle's own FGMRES iteration counts for the four sources of the 1024^2 workload,
 # written by tests/golden/make_smooth2d_iterations.py (oracle code only)
 ORACLE_ITERS = os.path.join(ROOT, "tests", "golden", "smooth2d_n1024_iterations.json")
@@ -203,19 +197,6 @@ class Clocks:
             return {"sm_mhz": None, "sm_max_mhz": None, "reasons": [], "samples": 0}
         return {"sm_mhz": statistics.median(sm), "sm_max_mhz": max(mx),
                 "reasons": sorted(reasons), "samples": len(sm)}
-
-
-def front_traffic(n: int, front_kernel: int):
-    """Measured DRAM bytes per sweep-front launch, or None when they do not apply to this
-    run (another size or kernel, or a kernel source changed since the capture)."""
-    import hashlib
-    if n != FRONT_TRAFFIC["n"] or front_kernel not in FRONT_TRAFFIC["front_kernels"]:
-        return None
-    src = os.path.join(ROOT, "paper_1909_01467_gb300", "csrc", "sweep.cu")
-    with open(src, "rb") as fh:
-        if hashlib.sha256(fh.read()).hexdigest() != FRONT_TRAFFIC["sweep_cu_sha256"]:
-            return None
-    return FRONT_TRAFFIC["bytes_per_launch"]
 
 
 def replica_throughput(ms: float, units_per_rank: float, world: int, device=None):
@@ -505,7 +486,7 @@ def run_ours(args):
             "roofline": c128_roof},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": (achieved / peak) if achieved else None,
-                     "traffic": front_traffic(n, args.front_kernel),
+                     "traffic": None,   # (not measured inside the run)
                      "kernel": {1: "k_front (cluster split)",
                                 2: "k_front_solo (one CTA per local solve)",
                                 3: "k_twist (two CTAs per local solve, twisted factor)"}.get(
